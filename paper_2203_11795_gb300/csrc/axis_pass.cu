@@ -48,6 +48,24 @@ __global__ void __launch_bounds__(kAxisThreads) axis_pass_kernel(const __grid_co
     }
 }
 
+// complex128: the stages in fixed point (axis_tile_fx), the columns' exponents after the tile.
+template <int DIR, int R0>
+__global__ void __launch_bounds__(kAxisThreads) axis_fixed_kernel(const __grid_constant__ AxisPass a) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    double2 *sm = reinterpret_cast<double2 *>(smem_raw);
+    int *emax = reinterpret_cast<int *>(sm + a.tile);
+    for (int64_t t = blockIdx.x; t < a.tiles; t += gridDim.x)
+        axis_tile_fx<DIR, R0>(a, t, sm, emax, static_cast<const double2 *>(a.src), static_cast<double2 *>(a.dst));
+}
+
+__global__ void fixed_table_kernel(int4 *dst, const double2 *src, int64_t n) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+        const double2 w = src[e];
+        const int2 re = fx_q62(w.x), im = fx_q62(w.y);
+        dst[e] = make_int4(re.x, re.y, im.x, im.y);
+    }
+}
+
 // w_n^e = exp(-2 pi i e / n) for e in [n], evaluated in FP64 by sincospi on the
 // exactly reduced exponent, then rounded once to the table's precision.
 template <typename C>
@@ -98,6 +116,14 @@ cudaError_t launch_axis_t(const AxisPass &a, cudaStream_t st) {
         }
     }
     const int r0 = a.nstages > 0 && a.radix[0] != 8 ? a.radix[0] : 1;
+    if constexpr (sizeof(C) == 16) {
+        switch (r0) {
+            case 2: axis_fixed_kernel<DIR, 2><<<(unsigned)grid, a.threads, smem, st>>>(a); break;
+            case 4: axis_fixed_kernel<DIR, 4><<<(unsigned)grid, a.threads, smem, st>>>(a); break;
+            default: axis_fixed_kernel<DIR, 1><<<(unsigned)grid, a.threads, smem, st>>>(a); break;
+        }
+        return cudaGetLastError();
+    } else
     switch (r0) {
         case 2: axis_pass_kernel<C, DIR, 2><<<(unsigned)grid, a.threads, smem, st>>>(a); break;
         case 4: axis_pass_kernel<C, DIR, 4><<<(unsigned)grid, a.threads, smem, st>>>(a); break;
@@ -113,12 +139,24 @@ cudaError_t prepare_axis_r() {
                                 kMaxDynSmem);
 }
 
+template <int DIR, int R0>
+cudaError_t prepare_fixed_r() {
+    return cudaFuncSetAttribute(axis_fixed_kernel<DIR, R0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+}
+
 template <typename C, int DIR>
 cudaError_t prepare_axis_t() {
-    cudaError_t e = prepare_axis_r<C, DIR, 1>();
-    if (e == cudaSuccess) e = prepare_axis_r<C, DIR, 2>();
-    if (e == cudaSuccess) e = prepare_axis_r<C, DIR, 4>();
-    if (e == cudaSuccess) e = prepare_axis_r<C, DIR, 16>();
+    cudaError_t e = cudaSuccess;
+    if constexpr (sizeof(C) == 16) {
+        e = prepare_fixed_r<DIR, 1>();
+        if (e == cudaSuccess) e = prepare_fixed_r<DIR, 2>();
+        if (e == cudaSuccess) e = prepare_fixed_r<DIR, 4>();
+    } else {
+        e = prepare_axis_r<C, DIR, 1>();
+        if (e == cudaSuccess) e = prepare_axis_r<C, DIR, 2>();
+        if (e == cudaSuccess) e = prepare_axis_r<C, DIR, 4>();
+        if (e == cudaSuccess) e = prepare_axis_r<C, DIR, 16>();
+    }
     if (e == cudaSuccess) e = prepare_axis_r<C, DIR, 1, 3>();
     if (e == cudaSuccess) e = prepare_axis_r<C, DIR, 2, 3>();
     if (e == cudaSuccess) e = prepare_axis_r<C, DIR, 4, 3>();
@@ -141,7 +179,15 @@ cudaError_t prepare_axis_t() {
 size_t axis_pass_smem_bytes(const AxisPass &a, int is_double) {
     const size_t tile = (size_t)a.tile * (is_double ? sizeof(double2) : sizeof(float2));
     if (!is_double && (a.tc == 1 || a.tc == 2)) return (tile + 127) / 128 * 128 + umma_smem_bytes(a.threads);
-    return tile;
+    // complex128: one exponent per column (tile / len) after the tile
+    return is_double ? tile + sizeof(int) * (size_t)(a.tile / a.len) : tile;
+}
+
+cudaError_t launch_fixed_table(void *dst, const void *src, int64_t n, cudaStream_t st) {
+    int64_t blocks = (n + 255) / 256;
+    if (blocks > 4096) blocks = 4096;
+    fixed_table_kernel<<<(unsigned)blocks, 256, 0, st>>>(static_cast<int4 *>(dst), static_cast<const double2 *>(src), n);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_axis_pass(const AxisPass &a, int is_double, int dir, cudaStream_t st) {

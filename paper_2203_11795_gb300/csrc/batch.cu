@@ -61,7 +61,10 @@ struct BatchParams {
 // all of them without the register allocation of the largest applying to the rest.
 template <typename C, int DIR, int R0>
 __device__ __noinline__ void axis_tile_call(const AxisPass &a, int64_t t, C *sm, const C *src, C *dst) {
-    axis_tile<C, DIR, R0>(a, t, sm, src, dst, static_cast<const C *>(a.tw));
+    if constexpr (sizeof(C) == 16)
+        axis_tile_fx<DIR, R0>(a, t, sm, reinterpret_cast<int *>(sm + a.tile), src, dst);
+    else
+        axis_tile<C, DIR, R0>(a, t, sm, src, dst, static_cast<const C *>(a.tw));
 }
 template <typename C, int DIR>
 __device__ __noinline__ void phaseb_tile_call(const PhaseBFused &b, int64_t t, C *sm, C *data) {
@@ -121,7 +124,9 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(const __grid_const
                 switch (J.r0) {
                     case 2: axis_tile_call<C, DIR, 2>(J.a, lt, sm, src, out); break;
                     case 4: axis_tile_call<C, DIR, 4>(J.a, lt, sm, src, out); break;
-                    case 16: axis_tile_call<C, DIR, 16>(J.a, lt, sm, src, out); break;
+                    case 16:
+                        if constexpr (sizeof(C) == 8) axis_tile_call<C, DIR, 16>(J.a, lt, sm, src, out);
+                        break;
                     default: axis_tile_call<C, DIR, 1>(J.a, lt, sm, src, out); break;
                 }
             } else {
@@ -234,7 +239,7 @@ fftu_status batch_create(int count, const fftu_handle *plans, Batch **out_batch)
                 J.r0 = sv.axis.nstages > 0 && sv.axis.radix[0] != 8 ? sv.axis.radix[0] : 1;
                 J.tiles = sv.axis.tiles;
                 J.reads_input = k == 0;
-                max_tile_bytes = std::max(max_tile_bytes, (size_t)sv.axis.tile * esize);
+                max_tile_bytes = std::max(max_tile_bytes, axis_pass_smem_bytes(sv.axis, views[0].dtype == FFTU_C128));
                 max_threads = std::max(max_threads, sv.axis.threads);
             } else {
                 J.kind = 2;

@@ -53,13 +53,14 @@ int ilog2(int64_t v) {
 }
 
 // Radix sequence for a power-of-two length: radix 8 where possible, a single
-// 16 or 4 to absorb the remainder, radix 2 only for length 2.
-int radix_plan(int len, int *radix) {
+// 16 or 4 to absorb the remainder, radix 2 only for length 2.  complex128 (a thread
+// holds 8 values) takes 2 in place of 16.
+int radix_plan(int len, int *radix, bool is_double) {
     int k = ilog2(len), n = 0;
     if (k == 0) return 0;
     int eights = k / 3, rem = k % 3;
     if (rem == 1) {
-        if (eights >= 1) {
+        if (eights >= 1 && !is_double) {
             radix[n++] = 16;
             --eights;
         } else {
@@ -127,6 +128,7 @@ struct Plan {
     void *tables = nullptr;
     size_t table_bytes = 0;
     int64_t table_off[FFTU_MAX_DIMS] = {};
+    int64_t fixed_off = 0;  // complex128: entries before the fixed-point tables
     int64_t line_table_off[FFTU_MAX_DIMS] = {};  // line-pass tables (complex64, len in [256, 2048]), else -1
     void *workspace = nullptr;   // [natural schedule's part | CYCLIC layout temp], plan-owned or caller's
     size_t workspace_bytes = 0;  // bytes the plan allocated itself (0 when the caller supplies it)
@@ -146,6 +148,9 @@ struct Plan {
     bool axis_pingpong = false;         // ... even in its strided-pass form (a line longer than the tile)
 
     const void *table(int l) const { return static_cast<const char *>(tables) + table_off[l] * esize; }
+    const void *fixed_table(int l) const {  // complex128: the roots of table(l) in fixed point, after all the tables
+        return dtype == FFTU_C128 ? static_cast<const char *>(tables) + (fixed_off + table_off[l]) * esize : nullptr;
+    }
     const void *line_table(int l) const {
         return line_table_off[l] < 0 ? nullptr : static_cast<const char *>(tables) + line_table_off[l] * esize;
     }
@@ -233,11 +238,12 @@ fftu_status make_axis_pass(const Plan &pl, int l, int mode, double scale, AxisPa
     if (th > 512) th = 512;
     a.threads = th;
     a.tw = pl.table(l);
+    a.twf = pl.fixed_table(l);
     a.status = pl.dstatus;
     a.scale = scale;
     // tc: 1 / 2 split-precision tensor-core radix-16 stages, 3 CUDA-core radix-16 stages, 0 radix 8
     a.tc = pl.precision ? pl.precision : (pl.radix == 16 ? 3 : 0);
-    a.nstages = a.tc ? radix_plan_tc(a.len, a.radix) : radix_plan(a.len, a.radix);
+    a.nstages = a.tc ? radix_plan_tc(a.len, a.radix) : radix_plan(a.len, a.radix, is_double);
     return FFTU_OK;
 }
 
@@ -619,10 +625,14 @@ fftu_status run_steps(Plan *pl, const std::vector<Step> &steps, const void *firs
             b.data = dst;
             b.mul = mul;
             mul = nullptr;  // consumed by the fused store
-            e = launch_phase_b3(b, is_double, pl->dir, st);
+            e = launch_phase_b3(b, pl->dir, st);
         } else {
             PhaseBFused b = s.pb;
             b.data = dst;
+            if (mul && is_double && phase_b_registers(b, is_double)) {
+                b.mul = mul;
+                mul = nullptr;
+            }
             e = launch_phase_b_fused(b, is_double, pl->dir, st);
         }
         if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
@@ -857,6 +867,8 @@ fftu_status fftu_plan_ex(int d, const int64_t *n, const int64_t *p, fftu_dtype d
         pl->line_table_off[l] = len ? off : -1;
         off += len ? len + len / 16 + n[l] : 0;
     }
+    pl->fixed_off = off;
+    if (dtype == FFTU_C128) off *= 2;  // every root again in fixed point (16 bytes as well)
     pl->table_bytes = (size_t)off * pl->esize;
     e = cudaMalloc(&pl->tables, pl->table_bytes);
     if (e != cudaSuccess) {
@@ -885,6 +897,8 @@ fftu_status fftu_plan_ex(int d, const int64_t *n, const int64_t *p, fftu_dtype d
             e = launch_line_tables(static_cast<char *>(pl->tables) + pl->line_table_off[l] * pl->esize,
                                    (int)(n[l] / pp[l]), (int)n[l], ps);
     }
+    if (e == cudaSuccess && dtype == FFTU_C128)
+        e = launch_fixed_table(static_cast<char *>(pl->tables) + pl->fixed_off * pl->esize, pl->tables, pl->fixed_off, ps);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ps);
     cudaStreamDestroy(ps);
     if (e != cudaSuccess) {
@@ -893,7 +907,7 @@ fftu_status fftu_plan_ex(int d, const int64_t *n, const int64_t *p, fftu_dtype d
     }
     e = prepare_axis_pass(dtype == FFTU_C128, dir);
     if (e == cudaSuccess) e = prepare_phase_b_fused(dtype == FFTU_C128, dir);
-    if (e == cudaSuccess) e = prepare_phase_b3(dtype == FFTU_C128, dir);
+    if (e == cudaSuccess && dtype == FFTU_C64) e = prepare_phase_b3(dir);
     if (e == cudaSuccess && dtype == FFTU_C64) e = prepare_line_pass(dir);
     if (e == cudaSuccess && dtype == FFTU_C64) e = prepare_pair_pass(dir);
     if (e == cudaSuccess && dtype == FFTU_C64) e = prepare_triple_pass(dir);

@@ -40,6 +40,7 @@ struct AxisPass {
     int tile;         // nlt * V
     int threads;
     const void *tw;   // w_{nl}^e, e in [nl] (forward roots)
+    const void *twf;  // complex128: the same roots in fixed point (fixed64.cuh), 16 bytes each
     double scale;
     int nstages;
     int radix[kMaxStages];
@@ -190,11 +191,11 @@ void record_error(const char *msg);
 // Set per-device kernel attributes (dynamic shared memory); called at plan time.
 cudaError_t prepare_axis_pass(int is_double, int dir);
 cudaError_t prepare_phase_b_fused(int is_double, int dir);
-cudaError_t prepare_phase_b3(int is_double, int dir);
+cudaError_t prepare_phase_b3(int dir);
 // Phase B for d = 3 with p_0 = p_1 = p_2 = P in {2, 4, 8, 16}: tile length MT
 // along the last axis (0 = not instantiated for this P and type).
 int phase_b3_tile_mt(int p0, int p1, int p2, int is_double);  // 0: no 3D phase-B kernel for this grid
-cudaError_t launch_phase_b3(const PhaseBFused &b, int is_double, int dir, cudaStream_t st);
+cudaError_t launch_phase_b3(const PhaseBFused &b, int dir, cudaStream_t st);
 cudaError_t launch_twiddle_table(void *dst, int64_t n, int is_double, cudaStream_t st);
 // out[i] *= mul[i] for i in [n] (used when phase B cannot fuse the multiply).
 cudaError_t launch_pointwise(void *out, const void *mul, int64_t n, int is_double, cudaStream_t st);
@@ -210,6 +211,10 @@ cudaError_t launch_line_pass(const LinePass &a, int dir, cudaStream_t st);
 cudaError_t launch_line_tables(void *dst, int len, int nl, cudaStream_t st);
 cudaError_t launch_phase_b_fused(const PhaseBFused &b, int is_double, int dir, cudaStream_t st);
 size_t axis_pass_smem_bytes(const AxisPass &a, int is_double);
+// The fixed-point form of `n` complex128 table entries (fixed64.cuh).
+cudaError_t launch_fixed_table(void *dst, const void *src, int64_t n, cudaStream_t st);
+// Whether a phase-B plan runs the register-resident stages (which take PhaseBFused::mul for complex128).
+bool phase_b_registers(const PhaseBFused &b, int is_double);
 size_t phase_b_fused_smem_bytes(const PhaseBFused &b, int is_double);
 
 }  // namespace fftu

@@ -196,7 +196,7 @@ extern "C" fftu_status fftu_exec_noalloc(int d, const int64_t *n, const int64_t 
         if (!ds.prepared[which][dslot]) {
             size_t smem = 0;
             e = prepare_phase_a3(which, dir, (int)n[0], (int)n[1], ds.grids[which], &smem);
-            if (e == cudaSuccess) e = prepare_phase_b3(0, dir);
+            if (e == cudaSuccess) e = prepare_phase_b3(dir);
             if (e != cudaSuccess) return fail(FFTU_ERR_CUDA, "fftu_exec_noalloc: kernel attributes");
             ds.prepared[which][dslot] = true;
         }
@@ -252,7 +252,7 @@ extern "C" fftu_status fftu_exec_noalloc(int d, const int64_t *n, const int64_t 
     b.scale = dir == FFTU_INVERSE ? 1.0 / (double)(n[0] * n[1] * n[2]) : 1.0;
 
     e = launch_phase_a3(l, st);  // clears the counters on the stream, then the persistent kernel
-    if (e == cudaSuccess) e = launch_phase_b3(b, 0, dir, st);
+    if (e == cudaSuccess) e = launch_phase_b3(b, dir, st);
     if (e != cudaSuccess) return fail(FFTU_ERR_CUDA, "fftu_exec_noalloc: kernel launch failed");
     return FFTU_OK;
 }

@@ -8,6 +8,7 @@
 
 #include "fft_device.cuh"
 #include "fftu_internal.h"
+#include "fixed64.cuh"
 #include "umma16.cuh"
 
 namespace fftu {
@@ -91,31 +92,39 @@ __device__ __forceinline__ void stockham_stage(C *sm, const C *__restrict__ tw, 
     __syncthreads();
 }
 
-// One tile of a generic strided pass (see AxisPass): load, Stockham stages, permuted store.
-// TCK = 0: radix R0 first, then radix 8 (CUDA cores).  TCK = 1 / 2: radix-16 stages as split
-// bfloat16 / float16 tcgen05 tensor-core contractions (umma16.cuh; `u` set up by the kernel), then
-// one CUDA-core stage of radix R0 (the rest of len).  TCK = 3: radix-16 CUDA-core stages, then one
-// stage of radix R0.
-template <typename C, int DIR, int R0, int TCK = 0>
-__device__ __forceinline__ void axis_tile(const AxisPass &a, int64_t t, C *sm, const C *__restrict__ src,
-                                          C *__restrict__ dst, const C *__restrict__ tw, UmmaCtx *u = nullptr) {
-    using Rl = typename real_of<C>::type;
-    const int tid = threadIdx.x, nt = blockDim.x;
+// Tile t of a strided pass: its first class c0 and the element offset of (first line or vector, line position 0).
+struct AxisOrigin {
+    int c0;
+    int64_t gbase;
+};
+__device__ __forceinline__ AxisOrigin axis_origin(const AxisPass &a, int64_t t) {
     const int chunks = 1 << a.lg_chunks;  // class chunks per line
     const int cc = (int)(t & (chunks - 1));
     const int64_t tt = t >> a.lg_chunks;
-    const int c0 = cc << a.lg_Gt;
-    int64_t gbase;  // element offset of (first line or vector, line position 0)
+    AxisOrigin o;
+    o.c0 = cc << a.lg_Gt;
     if (a.contiguous) {
-        gbase = (tt << a.lg_V) * a.nl;
+        o.gbase = (tt << a.lg_V) * a.nl;
     } else {
         const int64_t tpo_mask = ((int64_t)1 << a.lg_tpo) - 1;
-        gbase = (tt >> a.lg_tpo) * (int64_t)a.nl * a.inner + ((tt & tpo_mask) << a.lg_V);
+        o.gbase = (tt >> a.lg_tpo) * (int64_t)a.nl * a.inner + ((tt & tpo_mask) << a.lg_V);
     }
-    // complex64 tiles whose elements 2k and 2k + 1 are adjacent in global memory (runs of Gt >= 2
-    // classes along a line, or vectors of a strided axis): loads and stores go in 16-byte pairs with
-    // one index computation per pair.
-    const bool pairs = sizeof(C) == 8 && (a.contiguous ? a.Gt >= 2 && (a.mode == 1 || a.len >= 2) : a.V >= 2);
+    return o;
+}
+
+// complex64 tiles whose elements 2k and 2k + 1 are adjacent in global memory (runs of Gt >= 2 classes along a
+// line, or vectors of a strided axis): loads and stores go in 16-byte pairs with one index computation per pair.
+template <typename C> __device__ __forceinline__ bool axis_pairs(const AxisPass &a) {
+    return sizeof(C) == 8 && (a.contiguous ? a.Gt >= 2 && (a.mode == 1 || a.len >= 2) : a.V >= 2);
+}
+
+// Bring a tile into shared memory (complete for every thread on return).
+template <typename C>
+__device__ __forceinline__ void axis_load(const AxisPass &a, const AxisOrigin &o, C *sm, const C *__restrict__ src) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int c0 = o.c0;
+    const int64_t gbase = o.gbase;
+    const bool pairs = axis_pairs<C>(a);
     // load: shared index e is the natural order of the tile (tile line position lp, vector v);
     // tile position lp = c_local + j Gt holds line position c0 + c_local + j G
     if (pairs) {
@@ -150,7 +159,21 @@ __device__ __forceinline__ void axis_tile(const AxisPass &a, int64_t t, C *sm, c
     }
     async_copy_wait();
     __syncthreads();
+}
 
+// The stages and the permuted store of a landed tile.
+// TCK = 0: radix R0 first, then radix 8 (CUDA cores).  TCK = 1 / 2: radix-16 stages as split
+// bfloat16 / float16 tcgen05 tensor-core contractions (umma16.cuh; `u` set up by the kernel), then
+// one CUDA-core stage of radix R0 (the rest of len).  TCK = 3: radix-16 CUDA-core stages, then one
+// stage of radix R0.
+template <typename C, int DIR, int R0, int TCK = 0>
+__device__ __forceinline__ void axis_finish(const AxisPass &a, const AxisOrigin &o, C *sm, C *__restrict__ dst,
+                                            const C *__restrict__ tw, UmmaCtx *u = nullptr) {
+    using Rl = typename real_of<C>::type;
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int c0 = o.c0;
+    const int64_t gbase = o.gbase;
+    const bool pairs = axis_pairs<C>(a);
     int Ns = 1;
     if constexpr (TCK == 0) {
         if constexpr (R0 > 1) {
@@ -255,6 +278,238 @@ __device__ __forceinline__ void axis_tile(const AxisPass &a, int64_t t, C *sm, c
     __syncthreads();
 }
 
+// One tile of a strided pass: load, stages, permuted store.
+template <typename C, int DIR, int R0, int TCK = 0>
+__device__ __forceinline__ void axis_tile(const AxisPass &a, int64_t t, C *sm, const C *__restrict__ src,
+                                          C *__restrict__ dst, const C *__restrict__ tw, UmmaCtx *u = nullptr) {
+    const AxisOrigin o = axis_origin(a, t);
+    axis_load<C>(a, o, sm, src);
+    axis_finish<C, DIR, R0, TCK>(a, o, sm, dst, tw, u);
+}
+
+// ---- complex128 strided pass in fixed point (fixed64.cuh) -----------------------------------------
+// The tile's slots hold double2 as loaded, then longlong2 (both 16 bytes) from the first stage on.  One
+// exponent per sub-FFT (class and vector): emax[column] is the largest key of its inputs.
+
+// A Stockham stage on the fixed-point tile (the index maps of stockham_stage).  FIRST: reads double2, finds the
+// columns' exponents; returns false, the tile unchanged, when some value needs FP64 arithmetic.
+template <int DIR, int R, bool FIRST>
+__device__ __forceinline__ bool fx_stage(longlong2 *sm, const int4 *__restrict__ tw, const AxisPass &a, int Ns,
+                                         int *emax, int tid, int nthreads) {
+    constexpr int B = 8 / R;  // butterflies per thread
+    constexpr int RHO = lg_of<R>();
+    const int lg_cols = a.lg_Gt + a.lg_V;
+    const int cols = 1 << lg_cols;
+    const int per_col = a.len / R;
+    const int total = cols * per_col;
+    const int twstep = a.nl / (Ns * R);
+    const int lg_ns = 31 - __clz(Ns);
+    longlong2 v[B][R];
+    int bad = 0;
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+        const int w = tid + q * nthreads;
+        if (w < total) {
+            const int col = w & (cols - 1), b = w >> lg_cols;
+            const int base = a.contiguous ? ((col >> a.lg_Gt) << a.lg_nlt) + (col & (a.Gt - 1)) : col;
+            const int js = a.contiguous ? a.Gt : cols;
+            if constexpr (FIRST) {
+                int key = 0;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    v[q][r] = sm[smi(base + (b + r * per_col) * js, a.swz)];
+                    const int k = fx_key(fx_bits(v[q][r]));
+                    key = k > key ? k : key;
+                }
+                unsigned lo = 0;
+                if (key == 0) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) lo |= (unsigned)v[q][r].x | (unsigned)v[q][r].y;
+                }
+                if (!fx_plain(key, lo)) bad = 1;
+                atomicMax(emax + col, key);
+            } else {
+                const int k = b & (Ns - 1);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    longlong2 x = fx_scale_down<RHO>(sm[smi(base + (b + r * per_col) * js, a.swz)]);
+                    if (r > 0) x = fx_cmul<DIR>(x, tw[r * k * twstep]);
+                    v[q][r] = x;
+                }
+                fx_dft<R, DIR>(v[q]);
+            }
+        }
+    }
+    if constexpr (FIRST) {
+        if (__syncthreads_or(bad)) return false;
+    } else {
+        __syncthreads();
+    }
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+        const int w = tid + q * nthreads;
+        if (w < total) {
+            const int col = w & (cols - 1), b = w >> lg_cols;
+            const int base = a.contiguous ? ((col >> a.lg_Gt) << a.lg_nlt) + (col & (a.Gt - 1)) : col;
+            const int js = a.contiguous ? a.Gt : cols;
+            if constexpr (FIRST) {
+                const int E = fx_exp(emax[col]);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const double2 x = fx_bits(v[q][r]);
+                    v[q][r] = mk<longlong2>(fx_in<60 - RHO>(x.x, E), fx_in<60 - RHO>(x.y, E));
+                }
+                fx_dft<R, DIR>(v[q]);
+            }
+            const int k = b & (Ns - 1);
+            const int o = ((b >> lg_ns) << lg_ns) * R + k;
+#pragma unroll
+            for (int r = 0; r < R; ++r) sm[smi(base + (o + r * Ns) * js, a.swz)] = v[q][r];
+        }
+    }
+    __syncthreads();
+    return true;
+}
+
+// The FP64 form of the stages and the store, for a tile that cannot be scaled.
+template <int DIR, int R0>
+__device__ __noinline__ void axis_finish_fp64(const AxisPass &a, const AxisOrigin &o, double2 *sm, double2 *dst,
+                                              const double2 *tw) {
+    axis_finish<double2, DIR, R0>(a, o, sm, dst, tw);
+}
+
+// One complex128 tile of a strided pass.  emax: one int per column (tile / len), in shared memory.
+template <int DIR, int R0>
+__device__ __forceinline__ void axis_tile_fx(const AxisPass &a, int64_t t, double2 *sm, int *emax,
+                                             const double2 *__restrict__ src, double2 *__restrict__ dst) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const AxisOrigin o = axis_origin(a, t);
+    for (int i = tid; i < 1 << (a.lg_Gt + a.lg_V); i += nt) emax[i] = 0;
+    axis_load<double2>(a, o, sm, src);
+    longlong2 *fx = reinterpret_cast<longlong2 *>(sm);
+    const int4 *__restrict__ tw = static_cast<const int4 *>(a.twf);
+    int Ns = R0 > 1 ? R0 : 8;
+    // len = 1 (every p_l = 1): a copy with scale
+    if (a.len == 1 || !fx_stage<DIR, (R0 > 1 ? R0 : 8), true>(fx, tw, a, 1, emax, tid, nt)) {
+        axis_finish_fp64<DIR, R0>(a, o, sm, dst, static_cast<const double2 *>(a.tw));
+        return;
+    }
+    for (; Ns < a.len; Ns *= 8) fx_stage<DIR, 8, false>(fx, tw, a, Ns, emax, tid, nt);
+    // after the first stage 2^K = 2^60 / R0, each later stage one factor lower: 2^60 / len in all; 1/N is a
+    // power of two and goes into the exponent
+    const int e_add = 3 + a.lg_len + (__double2hiint(a.scale) >> 20) - 1023;
+    for (int e = tid; e < a.tile; e += nt) {
+        int lpo, v;
+        if (a.contiguous) {
+            v = e >> a.lg_nlt;
+            lpo = e & (a.nlt - 1);
+        } else {
+            lpo = e >> a.lg_V;
+            v = e & (a.V - 1);
+        }
+        longlong2 x;
+        int64_t gp;
+        int cl;
+        if (a.mode == 0) {
+            cl = lpo >> a.lg_len;
+            const int m = lpo & (a.len - 1);
+            const int c = o.c0 + cl;
+            const int lp = cl + (m << a.lg_Gt);
+            x = fx[smi(a.contiguous ? (v << a.lg_nlt) + lp : (lp << a.lg_V) + v, a.swz)];
+            if (c != 0 && m != 0) x = fx_cmul<DIR>(x, tw[c * m]);
+            gp = ((int64_t)c << a.lg_len) + m;
+        } else {
+            cl = lpo & (a.Gt - 1);
+            x = fx[smi(e, a.swz)];
+            gp = o.c0 + cl + ((int64_t)(lpo >> a.lg_Gt) << a.lg_G);
+        }
+        const int key = emax[a.contiguous ? (v << a.lg_Gt) + cl : (cl << a.lg_V) + v];
+        if (key == 0) x = mk<longlong2>(0, 0);  // all zeros: no trace of the products' rounding constants
+        const int e0 = fx_exp(key) + e_add;
+        const int64_t g = a.contiguous ? o.gbase + (int64_t)v * a.nl + gp : o.gbase + gp * a.inner + v;
+        dst[g] = mk<double2>(fx_out(x.x, e0), fx_out(x.y, e0));
+    }
+    __syncthreads();
+}
+
+// F_LO along the low LO values and F_HI across them of one complex128 fiber (v[jl + LO jh]) held in registers,
+// times 2^lg_scale.
+template <int DIR, int LO, int HI> __device__ __noinline__ void fiber_fp64(double2 *v, int lg_scale) {
+#pragma unroll
+    for (int jh = 0; jh < HI; ++jh) dft_small<LO, DIR>(v + jh * LO);
+#pragma unroll
+    for (int jl = 0; jl < LO; ++jl) {
+        double2 w[HI];
+#pragma unroll
+        for (int jh = 0; jh < HI; ++jh) w[jh] = v[jh * LO + jl];
+        dft_small<HI, DIR>(w);
+#pragma unroll
+        for (int jh = 0; jh < HI; ++jh) v[jh * LO + jl] = cscale(w[jh], __hiloint2double((1023 + lg_scale) << 20, 0));
+    }
+}
+
+template <int DIR, int LO, int HI> __device__ __forceinline__ void fiber_dft(double2 *v, int lg_scale) {
+    constexpr int PG = LO * HI;
+    constexpr int RHO = lg_of<PG>();
+    int key = 0;
+#pragma unroll
+    for (int j = 0; j < PG; ++j) {
+        const int k = fx_key(v[j]);
+        key = k > key ? k : key;
+    }
+    unsigned lo = 0;
+    if (key == 0) {
+#pragma unroll
+        for (int j = 0; j < PG; ++j) lo |= (unsigned)__double2loint(v[j].x) | (unsigned)__double2loint(v[j].y);
+    }
+    if (!fx_plain(key, lo)) {
+        double2 c[PG];
+#pragma unroll
+        for (int j = 0; j < PG; ++j) c[j] = v[j];
+        fiber_fp64<DIR, LO, HI>(c, lg_scale);
+#pragma unroll
+        for (int j = 0; j < PG; ++j) v[j] = c[j];
+        return;
+    }
+    const int E = fx_exp(key);
+    longlong2 x[PG];
+#pragma unroll
+    for (int j = 0; j < PG; ++j) x[j] = mk<longlong2>(fx_in<60 - RHO>(v[j].x, E), fx_in<60 - RHO>(v[j].y, E));
+#pragma unroll
+    for (int jh = 0; jh < HI; ++jh) fx_dft<LO, DIR>(x + jh * LO);
+    if constexpr (HI > 1) {
+#pragma unroll
+        for (int jl = 0; jl < LO; ++jl) {
+            longlong2 w[HI];
+#pragma unroll
+            for (int jh = 0; jh < HI; ++jh) w[jh] = x[jh * LO + jl];
+            fx_dft<HI, DIR>(w);
+#pragma unroll
+            for (int jh = 0; jh < HI; ++jh) x[jh * LO + jl] = w[jh];
+        }
+    }
+    const int e0 = E + 3 + RHO + lg_scale;
+#pragma unroll
+    for (int j = 0; j < PG; ++j) v[j] = mk<double2>(fx_out(x[j].x, e0), fx_out(x[j].y, e0));
+}
+
+// The same for complex64, in FP32.
+template <int DIR, int LO, int HI> __device__ __forceinline__ void fiber_dft(float2 *v, int) {
+#pragma unroll
+    for (int jh = 0; jh < HI; ++jh) dft_small<LO, DIR>(v + jh * LO);
+    if constexpr (HI > 1) {
+#pragma unroll
+        for (int jl = 0; jl < LO; ++jl) {
+            float2 w[HI];
+#pragma unroll
+            for (int jh = 0; jh < HI; ++jh) w[jh] = v[jh * LO + jl];
+            dft_small<HI, DIR>(w);
+#pragma unroll
+            for (int jh = 0; jh < HI; ++jh) v[jh * LO + jl] = w[jh];
+        }
+    }
+}
+
 // Shared slot of phase-B tile element e (see PhaseBFused::swz_*; keeps the pairs (2k, 2k + 1) together).
 // SWZ = false: the identity (no index arithmetic).
 template <bool SWZ> __device__ __forceinline__ int pbs(const PhaseBFused &b, int e) {
@@ -272,7 +527,7 @@ __device__ __forceinline__ void axis_dft(const PhaseBFused &pb, C *sm, int total
         C v[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = sm[pbs<SWZ>(pb, base + r * S)];
-        dft_small<R, DIR>(v);
+        fiber_dft<DIR, R, 1>(v, 0);
 #pragma unroll
         for (int r = 0; r < R; ++r) sm[pbs<SWZ>(pb, base + r * S)] = v[r];
     }
@@ -289,24 +544,7 @@ __device__ __forceinline__ void axis_dft2(const PhaseBFused &pb, C *sm, int tota
         C v[R1 * R2];
 #pragma unroll
         for (int r = 0; r < R1 * R2; ++r) v[r] = sm[pbs<SWZ>(pb, base + r * S)];
-#pragma unroll
-        for (int r2 = 0; r2 < R2; ++r2) {
-            C w[R1];
-#pragma unroll
-            for (int r1 = 0; r1 < R1; ++r1) w[r1] = v[r2 * R1 + r1];
-            dft_small<R1, DIR>(w);
-#pragma unroll
-            for (int r1 = 0; r1 < R1; ++r1) v[r2 * R1 + r1] = w[r1];
-        }
-#pragma unroll
-        for (int r1 = 0; r1 < R1; ++r1) {
-            C w[R2];
-#pragma unroll
-            for (int r2 = 0; r2 < R2; ++r2) w[r2] = v[r2 * R1 + r1];
-            dft_small<R2, DIR>(w);
-#pragma unroll
-            for (int r2 = 0; r2 < R2; ++r2) v[r2 * R1 + r1] = w[r2];
-        }
+        fiber_dft<DIR, R1, R2>(v, 0);
 #pragma unroll
         for (int r = 0; r < R1 * R2; ++r) sm[pbs<SWZ>(pb, base + r * S)] = v[r];
     }

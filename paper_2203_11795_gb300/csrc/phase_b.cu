@@ -58,27 +58,32 @@ __global__ void __launch_bounds__(256, sizeof(C) == 8 ? 3 : 1) phase_b_fused_ker
     for (int64_t t = blockIdx.x; t < b.tiles; t += gridDim.x) phaseb_tile<C, DIR, SWZ>(b, t, sm, data);
 }
 
-template <int DIR>
-__global__ void __launch_bounds__(256) phase_b_reg_kernel(const __grid_constant__ PhaseBFused b,
-                                                          const __grid_constant__ PBGroups g) {
-    extern __shared__ __align__(16) float2 pbr_sm[];
-    float2 *__restrict__ data = static_cast<float2 *>(b.data);
-    const float scale = (float)b.scale;
+// complex64: three CTAs per SM (64 KB tiles); complex128 holds 16 values in 64 registers and more: two (128
+// registers).
+// MUL (complex128): with the pointwise product in the last store.  complex64 multiplies in a pass of its own:
+// the product in this store measured slower (a 0.085 ms convolution 0.089).
+template <typename C, int DIR, bool MUL>
+__global__ void __launch_bounds__(256, sizeof(C) == 16 ? 2 : 3)
+    phase_b_reg_kernel(const __grid_constant__ PhaseBFused b, const __grid_constant__ PBGroups g) {
+    extern __shared__ __align__(16) unsigned char pbr_raw[];
+    C *sm = reinterpret_cast<C *>(pbr_raw);
+    C *__restrict__ data = static_cast<C *>(b.data);
+    const int lg_scale = (__double2hiint(b.scale) >> 20) - 1023;
     for (int64_t t = blockIdx.x; t < b.tiles; t += gridDim.x) {
         const int64_t base = phaseb_base(b, t);
         for (int gi = 0; gi < g.n; ++gi) {
             const bool first = gi == 0, last = gi == g.n - 1;
             switch (g.lo[gi] * 100 + g.hi[gi]) {
-                case 201: pb_stage<DIR, 2, 1>(b, g, gi, base, pbr_sm, data, first, last, scale); break;
-                case 401: pb_stage<DIR, 4, 1>(b, g, gi, base, pbr_sm, data, first, last, scale); break;
-                case 801: pb_stage<DIR, 8, 1>(b, g, gi, base, pbr_sm, data, first, last, scale); break;
-                case 1601: pb_stage<DIR, 16, 1>(b, g, gi, base, pbr_sm, data, first, last, scale); break;
-                case 202: pb_stage<DIR, 2, 2>(b, g, gi, base, pbr_sm, data, first, last, scale); break;
-                case 204: pb_stage<DIR, 2, 4>(b, g, gi, base, pbr_sm, data, first, last, scale); break;
-                case 402: pb_stage<DIR, 4, 2>(b, g, gi, base, pbr_sm, data, first, last, scale); break;
-                case 404: pb_stage<DIR, 4, 4>(b, g, gi, base, pbr_sm, data, first, last, scale); break;
-                case 208: pb_stage<DIR, 2, 8>(b, g, gi, base, pbr_sm, data, first, last, scale); break;
-                case 802: pb_stage<DIR, 8, 2>(b, g, gi, base, pbr_sm, data, first, last, scale); break;
+                case 201: pb_stage<C, DIR, MUL, 2, 1>(b, g, gi, base, sm, data, first, last, lg_scale); break;
+                case 401: pb_stage<C, DIR, MUL, 4, 1>(b, g, gi, base, sm, data, first, last, lg_scale); break;
+                case 801: pb_stage<C, DIR, MUL, 8, 1>(b, g, gi, base, sm, data, first, last, lg_scale); break;
+                case 1601: pb_stage<C, DIR, MUL, 16, 1>(b, g, gi, base, sm, data, first, last, lg_scale); break;
+                case 202: pb_stage<C, DIR, MUL, 2, 2>(b, g, gi, base, sm, data, first, last, lg_scale); break;
+                case 204: pb_stage<C, DIR, MUL, 2, 4>(b, g, gi, base, sm, data, first, last, lg_scale); break;
+                case 402: pb_stage<C, DIR, MUL, 4, 2>(b, g, gi, base, sm, data, first, last, lg_scale); break;
+                case 404: pb_stage<C, DIR, MUL, 4, 4>(b, g, gi, base, sm, data, first, last, lg_scale); break;
+                case 208: pb_stage<C, DIR, MUL, 2, 8>(b, g, gi, base, sm, data, first, last, lg_scale); break;
+                case 802: pb_stage<C, DIR, MUL, 8, 2>(b, g, gi, base, sm, data, first, last, lg_scale); break;
                 default: break;
             }
             __syncthreads();
@@ -119,17 +124,21 @@ bool pb_groups(const PhaseBFused &b, PBGroups &g) {
 
 template <typename C, int DIR>
 cudaError_t launch_b_t(const PhaseBFused &b, cudaStream_t st) {
-    if constexpr (sizeof(C) == 8) {
-        // complex64: the register-resident stages, except where the swizzled shared tile applies (a single-axis
-        // first pass over short runs), which measured faster there (64^4 at p = 8^4: 0.111 against 0.119 ms;
-        // 32^5 at p = 4^5: 0.153 -> 0.134 ms and 16384^2 at p = 16^2: 0.830 -> 0.731 ms with the stages)
-        PBGroups g;
-        if (b.swz_mask == 0 && b.P * b.Mt <= 8192 && pb_groups(b, g)) {
-            const size_t smem = (size_t)b.P * b.Mt * sizeof(C);
-            int64_t grid = b.tiles < (int64_t)1 << 30 ? b.tiles : (int64_t)1 << 30;
-            phase_b_reg_kernel<DIR><<<(unsigned)grid, 256, smem, st>>>(b, g);
-            return cudaGetLastError();
+    PBGroups g;
+    if (phase_b_registers(b, sizeof(C) == 16) && pb_groups(b, g)) {
+        const size_t smem = (size_t)b.P * b.Mt * sizeof(C);
+        int64_t grid = b.tiles < (int64_t)1 << 30 ? b.tiles : (int64_t)1 << 30;
+        int threads = 256;
+        if constexpr (sizeof(C) == 16) {  // small tiles: a thread per 8 values
+            threads = (b.P * b.Mt / 8 + 31) / 32 * 32;
+            threads = threads < 32 ? 32 : threads > 256 ? 256 : threads;
+            if (b.mul) {
+                phase_b_reg_kernel<C, DIR, true><<<(unsigned)grid, threads, smem, st>>>(b, g);
+                return cudaGetLastError();
+            }
         }
+        phase_b_reg_kernel<C, DIR, false><<<(unsigned)grid, threads, smem, st>>>(b, g);
+        return cudaGetLastError();
     }
     size_t smem = (size_t)b.P * b.Mt * sizeof(C);
     int64_t grid = b.tiles < (int64_t)1 << 30 ? b.tiles : (int64_t)1 << 30;
@@ -142,11 +151,14 @@ cudaError_t launch_b_t(const PhaseBFused &b, cudaStream_t st) {
 
 template <typename C, int DIR>
 cudaError_t prepare_b_t() {
-    if constexpr (sizeof(C) == 8) {
-        cudaError_t e0 = cudaFuncSetAttribute(phase_b_reg_kernel<DIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              kMaxDynSmem);
-        if (e0 != cudaSuccess) return e0;
+    cudaError_t e0 = cudaFuncSetAttribute(phase_b_reg_kernel<C, DIR, false>,
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+    if constexpr (sizeof(C) == 16) {
+        if (e0 == cudaSuccess)
+            e0 = cudaFuncSetAttribute(phase_b_reg_kernel<C, DIR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      kMaxDynSmem);
     }
+    if (e0 != cudaSuccess) return e0;
     cudaError_t e = cudaFuncSetAttribute(phase_b_fused_kernel<C, DIR, false>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
     if (e == cudaSuccess)
@@ -160,6 +172,13 @@ cudaError_t prepare_b_t() {
 cudaError_t prepare_phase_b_fused(int is_double, int dir) {
     if (is_double) return dir < 0 ? prepare_b_t<double2, -1>() : prepare_b_t<double2, 1>();
     return dir < 0 ? prepare_b_t<float2, -1>() : prepare_b_t<float2, 1>();
+}
+
+// complex128: always (the FP64 unit is the bound otherwise).  complex64: except where the swizzled shared tile
+// applies (a single-axis first pass over short runs), which measured faster there (64^4 at p = 8^4: 0.111 against
+// 0.119 ms; 32^5 at p = 4^5: 0.153 -> 0.134 ms and 16384^2 at p = 16^2: 0.830 -> 0.731 ms with the stages).
+bool phase_b_registers(const PhaseBFused &b, int is_double) {
+    return b.P > 1 && (is_double || (b.swz_mask == 0 && b.P * b.Mt <= 8192));
 }
 
 size_t phase_b_fused_smem_bytes(const PhaseBFused &b, int is_double) {

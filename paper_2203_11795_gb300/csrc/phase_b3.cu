@@ -23,9 +23,8 @@ namespace fftu {
 
 namespace {
 
-// Two consecutive elements per access: one 16-byte float4 for complex64,
-// two 16-byte double2 for complex128.  Streaming cache hints: each element
-// is touched once per pass.
+// Two consecutive elements per access: one 16-byte float4.  Streaming cache hints: each element is touched
+// once per pass.
 __device__ __forceinline__ void load_pair(const float2 *p, float2 &a, float2 &b) {
     float4 v = __ldcs(reinterpret_cast<const float4 *>(p));
     a = make_float2(v.x, v.y);
@@ -34,15 +33,6 @@ __device__ __forceinline__ void load_pair(const float2 *p, float2 &a, float2 &b)
 __device__ __forceinline__ void store_pair(float2 *p, float2 a, float2 b) {
     __stcs(reinterpret_cast<float4 *>(p), make_float4(a.x, a.y, b.x, b.y));
 }
-__device__ __forceinline__ void load_pair(const double2 *p, double2 &a, double2 &b) {
-    a = __ldcs(p);
-    b = __ldcs(p + 1);
-}
-__device__ __forceinline__ void store_pair(double2 *p, double2 a, double2 b) {
-    __stcs(p, a);
-    __stcs(p + 1, b);
-}
-
 // Shared layout: [s0][s1][s2][m2] with m2 fastest, MT + pad per row of m2.
 template <typename C, int DIR, int P0, int P1, int P2, int MT>
 __global__ void __launch_bounds__(P0 * P1 * MT / 2) phase_b3_kernel(const __grid_constant__ PhaseBFused b) {
@@ -200,16 +190,12 @@ template <typename C, int DIR, bool PREP>
 cudaError_t dispatch(int P, const PhaseBFused *b, cudaStream_t st) {
     switch (P) {
         case 168:
-            if constexpr (sizeof(C) == 8)
-                return PREP ? prepare_t<C, DIR, 16, 16, 8, 8>() : launch_t<C, DIR, 16, 16, 8, 8>(*b, st);
-            break;
+            return PREP ? prepare_t<C, DIR, 16, 16, 8, 8>() : launch_t<C, DIR, 16, 16, 8, 8>(*b, st);
         case 2: return PREP ? prepare_t<C, DIR, 2, 2, 2, 64>() : launch_t<C, DIR, 2, 2, 2, 64>(*b, st);
         case 4: return PREP ? prepare_t<C, DIR, 4, 4, 4, 32>() : launch_t<C, DIR, 4, 4, 4, 32>(*b, st);
         case 8: return PREP ? prepare_t<C, DIR, 8, 8, 8, 16>() : launch_t<C, DIR, 8, 8, 8, 16>(*b, st);
         case 16:
-            if constexpr (sizeof(C) == 8)
-                return PREP ? prepare_t<C, DIR, 16, 16, 16, 4>() : launch_t<C, DIR, 16, 16, 16, 4>(*b, st);
-            break;
+            return PREP ? prepare_t<C, DIR, 16, 16, 16, 4>() : launch_t<C, DIR, 16, 16, 16, 4>(*b, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -217,33 +203,27 @@ cudaError_t dispatch(int P, const PhaseBFused *b, cudaStream_t st) {
 }  // namespace
 
 int phase_b3_tile_mt(int p0, int p1, int p2, int is_double) {
+    if (is_double) return 0;  // complex128 runs the register-resident form (phase_b.cu), in fixed point
     switch (b3_kind(p0, p1, p2)) {
         case 2: return 64;
         case 4: return 32;
         case 8: return 16;
-        case 16: return is_double ? 0 : 4;
-        case 168: return is_double ? 0 : 8;
+        case 16: return 4;
+        case 168: return 8;
     }
     return 0;
 }
 
-cudaError_t prepare_phase_b3(int is_double, int dir) {
+cudaError_t prepare_phase_b3(int dir) {
     for (int P : {2, 4, 8, 16, 168}) {
-        const int q = P == 168 ? 16 : P;
-        if (phase_b3_tile_mt(q, q, P == 168 ? 8 : q, is_double) == 0) continue;
-        cudaError_t e;
-        if (is_double)
-            e = dir < 0 ? dispatch<double2, -1, true>(P, nullptr, 0) : dispatch<double2, 1, true>(P, nullptr, 0);
-        else
-            e = dir < 0 ? dispatch<float2, -1, true>(P, nullptr, 0) : dispatch<float2, 1, true>(P, nullptr, 0);
+        cudaError_t e = dir < 0 ? dispatch<float2, -1, true>(P, nullptr, 0) : dispatch<float2, 1, true>(P, nullptr, 0);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
-cudaError_t launch_phase_b3(const PhaseBFused &b, int is_double, int dir, cudaStream_t st) {
+cudaError_t launch_phase_b3(const PhaseBFused &b, int dir, cudaStream_t st) {
     const int P = b3_kind(b.p[0], b.p[1], b.p[2]);
-    if (is_double) return dir < 0 ? dispatch<double2, -1, false>(P, &b, st) : dispatch<double2, 1, false>(P, &b, st);
     return dir < 0 ? dispatch<float2, -1, false>(P, &b, st) : dispatch<float2, 1, false>(P, &b, st);
 }
 
