@@ -114,6 +114,39 @@ template <int DIR, typename C> __device__ __forceinline__ void dft16(C *v) {
         }
 }
 
+// Radix 32 as 8 x 4, in place: column DFTs F_8 over x[q + 4 j] (q in [4]), weights w_32^{q k}, then row DFTs F_4 over q;
+// output k + 8 t.
+template <int DIR, typename C> __device__ __forceinline__ void dft32(C *v) {
+    using R = typename real_of<C>::type;
+    // cos and sin of 2 pi e / 32, e = 0 .. 8
+    constexpr double c[9] = {1.0, 0.98078528040323044913, 0.92387953251128675613, 0.83146961230254523708,
+                             0.70710678118654752440, 0.55557023301960222474, 0.38268343236508977173,
+                             0.19509032201612826785, 0.0};
+    C y[4][8];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) y[q][j] = v[q + 4 * j];
+        dft8<DIR>(y[q]);
+    }
+#pragma unroll
+    for (int q = 1; q < 4; ++q)
+#pragma unroll
+        for (int k = 1; k < 8; ++k) {
+            const int e = q * k;  // 1 .. 21 thirty-seconds of a turn
+            const double co = e <= 8 ? c[e] : e <= 16 ? -c[16 - e] : -c[e - 16];
+            const double si = e <= 8 ? c[8 - e] : e <= 16 ? c[e - 8] : -c[24 - e];
+            if (e == 8) y[q][k] = mul_w4<DIR>(y[q][k]);
+            else y[q][k] = cmul(y[q][k], mk<C>(R(co), DIR * R(si)));
+        }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        bfly4<DIR>(y[0][k], y[1][k], y[2][k], y[3][k]);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) v[k + 8 * t] = y[t][k];
+    }
+}
+
 // Physical shared-memory slot of tile index i of the strided passes: bits 1-3 XORed with bits 4-6 when
 // the pass asks for it (swz = 14, contiguous passes; 0: identity).  A bijection on every 16-element group
 // that keeps the pairs (2k, 2k + 1) together, so that the class-strided accesses of contiguous lines
@@ -130,6 +163,8 @@ template <int R, int DIR, typename C> __device__ __forceinline__ void dft_small(
         dft8<DIR>(v);
     } else if constexpr (R == 16) {
         dft16<DIR>(v);
+    } else if constexpr (R == 32) {
+        dft32<DIR>(v);
     }
 }
 

@@ -84,21 +84,23 @@ int radix_plan_tc(int len, int *radix) {
 
 enum StepKind {
     STEP_AXIS = 1, STEP_PHASE_B_FUSED = 2, STEP_PHASE_B3 = 3, STEP_PHASE_A3 = 4, STEP_LINE = 5, STEP_PAIR = 6,
-    STEP_TRIPLE = 7
+    STEP_TRIPLE = 7, STEP_TILE = 8
 };
 
 struct Step {
     int kind;
-    AxisPass axis;   // STEP_LINE and STEP_PAIR keep the strided-pass form of the same axis (in place; batching)
-    AxisPass axis2;  // STEP_PAIR / STEP_TRIPLE: the strided-pass form of the next axis down (run after `axis`)
-    AxisPass axis3;  // STEP_TRIPLE: the strided-pass form of the third axis (run after `axis2`)
+    AxisPass axis;   // the other kinds keep the strided-pass form of the same axis (in place; batching)
+    AxisPass axis2;  // STEP_PAIR / STEP_TRIPLE / STEP_TILE: the strided-pass form of the next axis (run after `axis`)
+    AxisPass axis3;  // STEP_TRIPLE / STEP_TILE: the strided-pass form of the third axis (run after `axis2`)
     PhaseBFused pb;
     Phase3Launch a3;
     LinePass line;
     PairPass pair;
     TriplePass triple;
+    TilePass tile;
+    int tile_axes;   // STEP_TILE: axes of the pass (at most 3)
 
-    int passes() const { return kind == STEP_TRIPLE ? 3 : kind == STEP_PAIR ? 2 : 1; }
+    int passes() const { return kind == STEP_TRIPLE ? 3 : kind == STEP_PAIR ? 2 : kind == STEP_TILE ? tile_axes : 1; }
     const AxisPass &strided(int i) const { return i == 0 ? axis : i == 1 ? axis2 : axis3; }
     bool whole_lines() const {
         for (int i = 0; i < passes(); ++i)
@@ -142,7 +144,9 @@ struct Plan {
     int radix = 8;               // 8 or 16: stage radix of the strided passes
     int *dstatus = nullptr;
     int tuned = 0;
+    bool free_grid = false;      // the grid is the library's default: fftu_exec may take whole-axis passes
     std::vector<Step> phase_a, phase_b;
+    std::vector<TilePass> whole;  // fftu_exec: whole-axis passes in place of phase A and phase B (empty: not used)
     std::vector<Step> phase_a_inplace;  // used when in == out and phase_a cannot run in place
     bool generic_pingpong = false;      // generic phase A alternates between out and the workspace
     bool axis_pingpong = false;         // ... even in its strided-pass form (a line longer than the tile)
@@ -427,7 +431,59 @@ bool make_triple_pass(const Plan &pl, TriplePass &a) {
     return true;
 }
 
-fftu_status build_generic_phase_a(Plan &pl, std::vector<Step> &out, bool allow_line) {
+// The tile pass that ends at axis l1 of the d-dimensional array n (p: phase A on that grid; NULL: whole axes): as many
+// axes l0 .. l1 >= l_min as fit, and the vectors per tile.  Tiles of usually 4096 complex64 (32 KB, 256 threads) or
+// 2048 complex128 elements, up to 64 KB.  Runs on a strided group: complex64 16 elements (128 bytes), 8 where 16 do
+// not fit the tile; complex128 4.  Measured on 512 x 512 x 256 complex64 (floor 158 us a pass): the 512-point axes 214 and
+// 358 us at 8, 192 and 190 us at 16; a 1024-point axis 223-279 us at 8, 246-262 us at 16 with a 128 KB tile.
+bool choose_tile_pass(int d, const int64_t *n, const int64_t *p, int l1, int l_min, int is_double,
+                      const void *const *tw, const void *const *tw64, int *l0_out, TilePass &a) {
+    const int target = is_double ? 11 : 12, max_tile = is_double ? 12 : 13, min_v = is_double ? 2 : 3;
+    int64_t inner = 1, N = 1;
+    for (int l = 0; l < d; ++l) N *= n[l];
+    for (int l = l1 + 1; l < d; ++l) inner *= n[l];
+    const bool contiguous = inner == 1;
+    const int lg_in = ilog2(inner);
+    const int need_v = contiguous ? 0 : std::min(min_v, lg_in);
+    const int max_g = contiguous ? target : max_tile - need_v;  // several axes
+    int l0 = l1, lg_g = ilog2(n[l1]);
+    if (lg_g + need_v > max_tile) return false;
+    while (l0 > l_min && l1 - l0 < 2 && lg_g + ilog2(n[l0 - 1]) <= max_g) lg_g += ilog2(n[--l0]);
+    for (;; ++l0) {  // fewer axes when the stages do not work out
+        while (l0 < l1 && n[l0] == 1) ++l0;
+        int64_t outer = 1;
+        lg_g = 0;
+        for (int l = 0; l < l0; ++l) outer *= n[l];
+        for (int l = l0; l <= l1; ++l) lg_g += ilog2(n[l]);
+        int lg_v = std::max(target - lg_g, need_v);
+        if (!contiguous && !is_double && lg_v == 3 && lg_g + 4 <= max_tile) lg_v = 4;
+        lg_v = std::min(lg_v, contiguous ? ilog2(outer) : lg_in);
+        // small arrays: smaller tiles while the GPU is not full
+        while (lg_v > (contiguous ? 0 : need_v) && lg_v + lg_g > 9 && (N >> (lg_g + lg_v)) < 304) --lg_v;
+        if (make_tile_pass(d, n, p, l0, l1, is_double, 0, lg_v, tw, tw64, a)) {
+            // complex64: radix-32 stages where they save stages (1024-point contiguous lines 210 -> 172 us, strided
+            // 259 -> 223 us per 64 M elements).  Not on contiguous groups of several axes (32 x 32 planes: 3 stages 143
+            // us against 4 at 132), on single-stage contiguous lines (a thread per line scatters its accesses), or
+            // where 32 values a thread leave SMs idle (1024 x 1024: 18 against 11 us).
+            TilePass w;
+            if (!is_double && (N >> 22) > 0 && !(contiguous && l0 < l1) &&
+                make_tile_pass(d, n, p, l0, l1, 0, 1, lg_v, tw, tw64, w) && w.nst < a.nst && (w.nst > 1 || !contiguous))
+                a = w;
+            *l0_out = l0;
+            return true;
+        }
+        if (l0 == l1) return false;
+    }
+}
+
+// allow_line: passes that are never in place.  allow_tile: tile passes in place of strided ones.
+fftu_status build_generic_phase_a(Plan &pl, std::vector<Step> &out, bool allow_line, bool allow_tile) {
+    const int is_double = pl.dtype == FFTU_C128;
+    const void *tw[FFTU_MAX_DIMS], *tw64[FFTU_MAX_DIMS];
+    for (int l = 0; l < pl.d; ++l) {
+        tw[l] = is_double ? pl.fixed_table(l) : pl.table(l);
+        tw64[l] = is_double ? pl.table(l) : nullptr;
+    }
     // Contiguous axis first (reads the caller's array in long runs).  Out of place, two adjacent axes
     // with short sub-FFTs go through HBM once (pair pass); long sub-FFTs take the line pass.
     for (int l = pl.d - 1; l >= 0; --l) {
@@ -459,6 +515,26 @@ fftu_status build_generic_phase_a(Plan &pl, std::vector<Step> &out, bool allow_l
             continue;
         }
         if (allow_line && make_line_pass(pl, l, s.line)) s.kind = STEP_LINE;
+        int l0 = l, l_min = l;
+        if (s.kind == STEP_AXIS && allow_tile) {
+            // axes that a line or pair pass would not take can join
+            while (l_min > 0 && !(allow_line && line_len(pl.n, pl.p, l_min - 1, pl.dtype, pl.precision) > 0) &&
+                   !(allow_line && l_min > 1 && pl.n[l_min - 1] > 1 && pl.n[l_min - 2] > 1 &&
+                     make_pair_pass(pl, l_min - 1, s.pair)))
+                --l_min;
+            if (choose_tile_pass(pl.d, pl.n, pl.p, l, l_min, is_double, tw, tw64, &l0, s.tile)) {
+                cudaError_t e = prepare_tile_pass(s.tile, is_double, pl.dir);
+                if (e != cudaSuccess) return cuda_fail(e, "tile pass attributes");
+                s.kind = STEP_TILE;
+                s.tile_axes = 1;
+                for (int k = l - 1; k >= l0; --k) {
+                    if (pl.n[k] == 1) continue;
+                    st = make_axis_pass(pl, k, 0, 1.0, ++s.tile_axes == 2 ? s.axis2 : s.axis3);
+                    if (st != FFTU_OK) return st;
+                }
+                l = l0;
+            }
+        }
         out.push_back(s);
     }
     return FFTU_OK;
@@ -512,6 +588,39 @@ fftu_status build_fused_phase_a(Plan &pl, bool *used) {
     return FFTU_OK;
 }
 
+// The whole transform as passes over groups of whole axes (tile_pass.cuh), last axes first; no workspace.  Left
+// empty when some axis does not fit a tile.
+fftu_status build_whole(Plan &pl) {
+    const int is_double = pl.dtype == FFTU_C128;
+    int64_t n[FFTU_MAX_DIMS];
+    const void *tw[FFTU_MAX_DIMS], *tw64[FFTU_MAX_DIMS];
+    int d = 0;
+    for (int l = 0; l < pl.d; ++l) {
+        if (pl.n[l] == 1) continue;
+        n[d] = pl.n[l];
+        tw[d] = is_double ? pl.fixed_table(l) : pl.table(l);
+        tw64[d] = is_double ? pl.table(l) : nullptr;
+        ++d;
+    }
+    if (d == 0) return FFTU_OK;
+    std::vector<TilePass> steps;
+    for (int l1 = d - 1; l1 >= 0;) {
+        TilePass a;
+        int l0 = l1;
+        if (!choose_tile_pass(d, n, nullptr, l1, 0, is_double, tw, tw64, &l0, a)) return FFTU_OK;
+        cudaError_t e = prepare_tile_pass(a, is_double, pl.dir);
+        if (e != cudaSuccess) return cuda_fail(e, "tile pass attributes");
+        steps.push_back(a);
+        l1 = l0 - 1;
+    }
+    if (pl.dir == FFTU_INVERSE) {
+        steps.back().scale = 1.0 / (double)pl.N;
+        steps.back().lg_scale = -ilog2(pl.N);
+    }
+    pl.whole = steps;
+    return FFTU_OK;
+}
+
 fftu_status build_schedule(Plan &pl, int sched) {
     const double scale = pl.dir == FFTU_INVERSE ? 1.0 / (double)pl.N : 1.0;
     bool fused_a = false;
@@ -521,7 +630,8 @@ fftu_status build_schedule(Plan &pl, int sched) {
     }
     {
         // line passes are never in place: only the plain phase-A list takes them
-        fftu_status st = build_generic_phase_a(pl, fused_a ? pl.phase_a_inplace : pl.phase_a, !fused_a);
+        const bool tiles = (sched == FFTU_SCHED_AUTO || sched == FFTU_SCHED_FUSED) && pl.precision == FFTU_PREC_NATIVE;
+        fftu_status st = build_generic_phase_a(pl, fused_a ? pl.phase_a_inplace : pl.phase_a, !fused_a, tiles);
         if (st != FFTU_OK) return st;
     }
     if (!fused_a) {
@@ -530,7 +640,7 @@ fftu_status build_schedule(Plan &pl, int sched) {
         for (const Step &s : pl.phase_a) {
             const bool long_line = !s.whole_lines();
             if (long_line) pl.axis_pingpong = true;
-            if (s.kind != STEP_AXIS || long_line) pl.generic_pingpong = true;
+            if ((s.kind != STEP_AXIS && s.kind != STEP_TILE) || long_line) pl.generic_pingpong = true;
         }
         if (pl.generic_pingpong) pl.ws_natural = (size_t)pl.N * pl.esize;
     }
@@ -561,6 +671,13 @@ fftu_status build_schedule(Plan &pl, int sched) {
             if (st != FFTU_OK) return st;
             pl.phase_b.push_back(t);
         }
+    }
+    // the library's own choice of grid and schedule: the whole transform by whole-axis passes, except where the ring
+    // phase A applies
+    const bool ring = fused_a && pl.phase_a[0].a3.mode == 1;
+    if (pl.free_grid && sched == FFTU_SCHED_AUTO && pl.precision == FFTU_PREC_NATIVE && !ring) {
+        fftu_status st = build_whole(pl);
+        if (st != FFTU_OK) return st;
     }
     pl.schedule = sched == FFTU_SCHED_GENERIC ? FFTU_SCHED_GENERIC
                   : sched == FFTU_SCHED_GENERIC_A ? FFTU_SCHED_GENERIC_A : FFTU_SCHED_FUSED;
@@ -612,6 +729,11 @@ fftu_status run_steps(Plan *pl, const std::vector<Step> &steps, const void *firs
             a.src = src;
             a.dst = dst;
             e = launch_axis_pass(a, is_double, pl->dir, st);
+        } else if (s.kind == STEP_TILE) {
+            TilePass a = s.tile;
+            a.src = src;
+            a.dst = dst;
+            e = launch_tile_pass(a, is_double, pl->dir, st);
         } else if (s.kind == STEP_LINE || s.kind == STEP_PAIR || s.kind == STEP_TRIPLE) {
             record_error("internal: a register-resident pass outside the alternating phase-A schedule");
             return FFTU_ERR_INTERNAL;
@@ -815,6 +937,7 @@ fftu_status fftu_plan_ex(int d, const int64_t *n, const int64_t *p, fftu_dtype d
             return FFTU_ERR_UNSUPPORTED;
         }
     int tuned = 0;
+    bool free_grid = !p;
     if (!p) {  // measured tuning on request; otherwise wisdom for this problem, if the process has any
         fftu_options base;
         std::memset(&base, 0, sizeof(base));
@@ -822,7 +945,10 @@ fftu_status fftu_plan_ex(int d, const int64_t *n, const int64_t *p, fftu_dtype d
         base.schedule = sched;
         TuneChoice tc;
         if (opts && opts->tune ? autotune(d, n, dtype, dir, base, &tc) : wisdom_lookup(d, n, dtype, dir, base, &tc)) {
-            for (int l = 0; l < d; ++l) pp[l] = tc.p[l];
+            for (int l = 0; l < d; ++l) {
+                free_grid = free_grid && pp[l] == tc.p[l];  // another grid than the default: run that grid
+                pp[l] = tc.p[l];
+            }
             sched = tc.schedule;
             if (tc.tile) tile = tc.tile;
             if (tc.radix) radix = tc.radix;
@@ -844,6 +970,7 @@ fftu_status fftu_plan_ex(int d, const int64_t *n, const int64_t *p, fftu_dtype d
     pl->dtype = dtype;
     pl->dir = dir;
     pl->tuned = tuned;
+    pl->free_grid = free_grid;
     pl->precision = precision;
     pl->layout = layout;
     pl->workspace_mode = ws_mode;
@@ -958,8 +1085,24 @@ fftu_status fftu_plan(int d, const int64_t *n, const int64_t *p, fftu_dtype dtyp
 namespace fftu {
 namespace {
 
+// The whole transform by whole-axis passes; mul: optional pointwise factor of the result.
+fftu_status exec_whole(Plan *pl, const void *in, const void *mul, void *out, cudaStream_t st) {
+    const void *src = in;
+    for (size_t k = 0; k < pl->whole.size(); ++k) {
+        TilePass a = pl->whole[k];
+        a.src = src;
+        a.dst = out;
+        a.mul = k + 1 == pl->whole.size() ? mul : nullptr;
+        cudaError_t e = launch_tile_pass(a, pl->dtype == FFTU_C128, pl->dir, st);
+        if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
+        src = out;
+    }
+    return FFTU_OK;
+}
+
 // The transform on the natural view (every layout ends up here).
 fftu_status exec_natural(Plan *pl, fftu_phase phase, const void *in, void *out, cudaStream_t st) {
+    if (phase == FFTU_PHASE_ALL && !pl->whole.empty()) return exec_whole(pl, in, nullptr, out, st);
     if ((phase & FFTU_PHASE_A) && pl->generic_pingpong) {
         // buffers: pass k (of np) writes out when np - k is even, the workspace otherwise.  In place with
         // np odd, the first pass runs in place on out in its strided-pass form (whole lines only).
@@ -974,7 +1117,12 @@ fftu_status exec_natural(Plan *pl, fftu_phase phase, const void *in, void *out, 
                 return FFTU_ERR_UNSUPPORTED;
             }
             cudaError_t e;
-            if (dst == src) {  // the in-place first step: its strided passes, then the alternation continues
+            if (s.kind == STEP_TILE) {
+                TilePass a = s.tile;
+                a.src = src;
+                a.dst = dst;
+                e = launch_tile_pass(a, pl->dtype == FFTU_C128, pl->dir, st);
+            } else if (dst == src) {  // the in-place first step: its strided passes, then the alternation continues
                 e = cudaSuccess;
                 for (int i = 0; i < s.passes() && e == cudaSuccess; ++i) {
                     AxisPass a = s.strided(i);
@@ -1151,6 +1299,10 @@ fftu_status fftu_exec_pointwise(fftu_handle fwd, fftu_handle inv, const void *in
     const bool ring_inplace = in == tmp && pf->phase_a.size() == 1 && pf->phase_a[0].kind == STEP_PHASE_A3 &&
                               pf->phase_a[0].a3.mode == 1 && !pf->phase_a_inplace.empty();
     fftu_status s = FFTU_OK;
+    if (!pf->whole.empty()) {
+        s = exec_whole(pf, in, mul, tmp, st);
+        return s == FFTU_OK ? fftu_exec_phase(inv, FFTU_PHASE_ALL, tmp, out, stream) : s;
+    }
     if (pf->generic_pingpong) {
         s = fftu_exec_phase(fwd, FFTU_PHASE_A, in, tmp, stream);
     } else {

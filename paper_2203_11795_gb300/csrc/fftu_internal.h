@@ -126,6 +126,54 @@ struct PhaseBFused {
     int swz_src, swz_mask, swz_dst;
 };
 
+// Tile pass (see tile_pass.cuh): every position of axes l0 .. l1 for 2^lg_v adjacent inner (or, on contiguous memory,
+// outer) positions per tile.  Whole axes (the full F_{n_l}), or phase A on them (F_{n_l/p_l} on every class, twiddle,
+// Put).  May be in place.
+constexpr int kTpStages = 8, kTpFields = 8;
+struct BitField {
+    int sh, mask, dst;  // ((x >> sh) & mask) << dst
+};
+struct TileStage {
+    int lg_r, pos;      // radix 2^lg_r on tile bits [pos, pos + lg_r)
+    int tw_kind;        // 0: none; 1: w_{R T}^{r j} between the digits of an axis; 2: w_n^{k s} after the last digit of a
+                        // phase-A axis
+    int lo, lg_q;       // twiddle column q in [2^lg_q]: kind 1 j = tile bits [lo, lo + lg_q); kind 2 class s = tile bits
+                        // [lo, lo + lg_p) and the axis' bits above the digit
+    int lg_p, lg_step;  // kind 1: exponent r j 2^lg_step; kind 2: exponent (k_prev + r 2^lg_step) s
+    int nk;             // kind 2: k_prev = fields k[] of the bits above the digit
+    BitField k[2];
+    int tab;            // the table's place in shared memory (elements): entry (r, q) at tab + (r << lg_q) + q
+    const void *tw;     // w_n^e (complex128: in fixed point)
+    const void *tw64;   // complex128: w_n^e as double2
+    int rx[32];         // shared slot of r << pos
+};
+struct TilePass {
+    const void *src;
+    void *dst;
+    const void *mul;    // optional pointwise factor at the output's natural index
+    int64_t tiles;
+    int grid, threads;  // persistent grid
+    int wide;           // complex64: radix-32 stages
+    int lg_g, lg_v, lg_inner, lg_tile;  // lg_g: positions of the axes; lg_inner < 0: contiguous
+    int lg_dft;                         // log2 of the points of one sub-DFT
+    int in_bit, out_bit;                // element-offset bit of the first stage's and the last stage's digit
+    int nst, nlast, nout, ngroup;
+    int swz[2];
+    BitField last[kTpFields], out[kTpFields];  // last stage: thread index -> tile index, -> element offset
+    BitField group[kTpFields];                 // complex128: tile index -> exponent group (one per sub-DFT)
+    int lg_groups;
+    int lg_scale;
+    double scale;       // 2^lg_scale
+    size_t tab_off, emax_off, smem;
+    TileStage st[kTpStages];
+};
+// Describe a pass over axes l0 .. l1 of the d-dimensional array n; p: phase A on that grid (NULL: whole axes); tw /
+// tw64: root tables per axis.  false: not served.
+bool make_tile_pass(int d, const int64_t *n, const int64_t *p, int l0, int l1, int is_double, int wide, int lg_v,
+                    const void *const *tw, const void *const *tw64, TilePass &a);
+cudaError_t prepare_tile_pass(TilePass &a, int is_double, int dir);
+cudaError_t launch_tile_pass(const TilePass &a, int is_double, int dir, cudaStream_t st);
+
 // Fused 3D phase A (complex64): see phase_a3.cu.
 struct Phase3Info {
     int64_t unit_elems;  // elements of one residue unit (s0, s1)

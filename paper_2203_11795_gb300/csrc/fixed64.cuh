@@ -205,6 +205,6 @@ template <int RHO> __device__ __forceinline__ longlong2 fx_scale_down(longlong2 
     return mk<longlong2>((a.x + half) >> RHO, (a.y + half) >> RHO);
 }
 
-template <int R> __host__ __device__ constexpr int lg_of() { return R == 2 ? 1 : R == 4 ? 2 : R == 8 ? 3 : R == 16 ? 4 : 0; }
+template <int R> __host__ __device__ constexpr int lg_of() { return R == 2 ? 1 : R == 4 ? 2 : R == 8 ? 3 : R == 16 ? 4 : R == 32 ? 5 : 0; }
 
 }  // namespace fftu

@@ -1,0 +1,308 @@
+// Tile passes (tile_pass.cuh): kernel, launch, and the planner that splits a pass into stages.
+#include <cuda_runtime.h>
+
+#include <cstring>
+#include <utility>
+
+#include "fft_device.cuh"
+#include "fftu_internal.h"
+#include "tile_pass.cuh"
+
+namespace fftu {
+namespace {
+
+// Persistent: the twiddle tables are built once per CTA.  Registers: 64 for complex64 (two CTAs of 512 threads, four of
+// 256), 80 for complex128 (the bound of 768 threads; three CTAs of 256).
+template <int ARITH, int DIR, bool MUL>
+__global__ void __launch_bounds__(ARITH == kTpF32 ? 512 : ARITH == kTpF32w ? 256 : 768, ARITH == kTpFixed ? 1 : 2) tile_pass_kernel(const __grid_constant__ TilePass a) {
+    using T = tp_type<ARITH>;
+    using E = typename T::elem;
+    extern __shared__ __align__(128) unsigned char tp_raw[];
+    auto *sm = reinterpret_cast<typename T::work *>(tp_raw);
+    auto *tabs = reinterpret_cast<typename T::tw *>(tp_raw + a.tab_off);
+    int *emax = reinterpret_cast<int *>(tp_raw + a.emax_off);
+    tp_tables<ARITH>(a, tabs);
+    for (int64_t t = blockIdx.x; t < a.tiles; t += gridDim.x) {
+        __syncthreads();  // tables ready; the previous tile's last stage done with its slots and exponents
+        if constexpr (ARITH == kTpFixed) {
+            for (int i = threadIdx.x; i < 1 << a.lg_groups; i += blockDim.x) emax[i] = 0;
+            __syncthreads();
+        }
+        const int64_t base = tp_base(a, t);
+        const E *src = static_cast<const E *>(a.src) + base;
+        E *dst = static_cast<E *>(a.dst) + base;
+        if (!tp_run<ARITH, DIR, MUL>(a, sm, tabs, emax, src, dst)) {
+            if constexpr (ARITH == kTpFixed) tp_run_fp64<DIR, MUL>(a, reinterpret_cast<double2 *>(sm), src, dst);
+        }
+    }
+}
+
+int ilog2(int64_t v) {
+    int r = 0;
+    while ((int64_t(1) << r) < v) ++r;
+    return r;
+}
+
+// Digits of an axis of 2^bits points, highest first: at most 2^top points each, the larger ones first.
+int split_digits(int bits, int top, int *dig) {
+    const int k = (bits + top - 1) / top;
+    if (top == 3 && bits == 4) {  // complex128: a thread holds 8 values of the first stage
+        dig[0] = 3;
+        dig[1] = 1;
+        return 2;
+    }
+    for (int i = 0; i < k; ++i) dig[i] = bits / k + (i < bits % k ? 1 : 0);
+    return k;
+}
+
+// Rank over GF(2) of n vectors of m bits.
+int gf2_rank(int *v, int n) {
+    int rank = 0;
+    for (int b = 1; b < 16; b <<= 1) {
+        int p = -1;
+        for (int i = rank; i < n; ++i)
+            if (v[i] & b) {
+                p = i;
+                break;
+            }
+        if (p < 0) continue;
+        const int t = v[p];
+        v[p] = v[rank];
+        v[rank] = t;
+        for (int i = 0; i < n; ++i)
+            if (i != rank && (v[i] & b)) v[i] ^= v[rank];
+        ++rank;
+    }
+    return rank;
+}
+
+template <int ARITH, int DIR>
+cudaError_t launch_t(const TilePass &a, cudaStream_t st) {
+    int64_t grid = a.tiles < a.grid ? a.tiles : a.grid;
+    if (a.mul)
+        tile_pass_kernel<ARITH, DIR, true><<<(unsigned)grid, a.threads, a.smem, st>>>(a);
+    else
+        tile_pass_kernel<ARITH, DIR, false><<<(unsigned)grid, a.threads, a.smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+template <int ARITH, int DIR>
+cudaError_t prepare_t(TilePass &a) {
+    cudaError_t e = cudaFuncSetAttribute(tile_pass_kernel<ARITH, DIR, false>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(tile_pass_kernel<ARITH, DIR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kMaxDynSmem);
+    int dev = 0, sms = 0, per_sm = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tile_pass_kernel<ARITH, DIR, false>, a.threads, a.smem);
+    if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
+    a.grid = sms * per_sm;
+    return e;
+}
+
+}  // namespace
+
+bool make_tile_pass(int d, const int64_t *n, const int64_t *p, int l0, int l1, int is_double, int wide, int lg_v,
+                    const void *const *tw, const void *const *tw64, TilePass &a) {
+    std::memset(&a, 0, sizeof(a));
+    int64_t outer = 1, inner = 1, G = 1;
+    for (int l = 0; l < l0; ++l) outer *= n[l];
+    for (int l = l0; l <= l1; ++l) G *= n[l];
+    for (int l = l1 + 1; l < d; ++l) inner *= n[l];
+    if (outer * G * inner > ((int64_t)1 << 31)) return false;  // 32-bit element offsets within a tile
+    const bool contiguous = inner == 1;
+    a.lg_g = ilog2(G);
+    a.lg_v = lg_v;
+    a.lg_inner = contiguous ? -1 : ilog2(inner);
+    a.lg_tile = a.lg_g + lg_v;
+    if (a.lg_tile > 14) return false;
+    a.tiles = (contiguous ? outer : outer * inner) >> lg_v;
+    const int top = is_double ? 3 : wide ? 5 : 4;
+    a.wide = wide;
+    // stage order: the slowest axis' first digit, the other axes' digits, the slowest axis' remaining digits: the
+    // first and last stage then run across rows, with lanes along memory.  A contiguous group whose slowest axis
+    // has one digit gets it split, so that the last stage is not the contiguous axis' only digit.
+    struct Dig {
+        int axis, bits, pos;
+    } dg[kTpStages];
+    int order[kTpStages], nd = 0, no = 0;
+    int lo_of[FFTU_MAX_DIMS], lg_p[FFTU_MAX_DIMS], first_of[FFTU_MAX_DIMS], count_of[FFTU_MAX_DIMS];
+    int lo = contiguous ? 0 : lg_v;
+    for (int l = l1; l >= l0; --l) {
+        lg_p[l] = p ? ilog2(p[l]) : 0;
+        const int bits = ilog2(n[l]) - lg_p[l];
+        int dig[8];
+        int k = split_digits(bits, top, dig);
+        if (l == l0 && l1 > l0 && contiguous && k == 1 && bits >= 2) {
+            dig[1] = bits / 2;
+            dig[0] = bits - dig[1];
+            k = 2;
+        }
+        if (p && l0 == l1 && k == 1 && lg_p[l] > 0) {  // the Put moves s: loads and stores need a barrier between them
+            if (bits < 2) return false;
+            dig[1] = bits / 2;
+            dig[0] = bits - dig[1];
+            k = 2;
+        }
+        lo_of[l] = lo;
+        first_of[l] = nd;
+        count_of[l] = k;
+        a.lg_dft += bits;
+        int q = lo + lg_p[l] + bits;
+        for (int i = 0; i < k; ++i) {
+            if (nd >= kTpStages) return false;
+            q -= dig[i];
+            dg[nd++] = {l, dig[i], q};
+        }
+        lo += lg_p[l] + bits;
+    }
+    if (count_of[l0] > 0) order[no++] = first_of[l0];
+    for (int l = l1; l > l0; --l)
+        for (int i = 0; i < count_of[l]; ++i) order[no++] = first_of[l] + i;
+    for (int i = 1; i < count_of[l0]; ++i) order[no++] = first_of[l0] + i;
+    if (no == 0) return false;
+    if (no == 1 && p && l1 > l0) return false;  // (axes of length 2 beside it: left to the strided pass)
+    a.nst = no;
+    // output position of every tile bit (element-offset bits, relative to the tile's base): an axis' first (highest)
+    // digit holds the lowest bits of k; the class s goes above k
+    int out_bit[32], k_bit[kTpStages];
+    for (int b = 0; b < a.lg_tile; ++b) out_bit[b] = b;
+    for (int l = l1; l >= l0; --l) {
+        int k_at = 0;
+        for (int i = 0; i < count_of[l]; ++i) {
+            const Dig &g = dg[first_of[l] + i];
+            k_bit[first_of[l] + i] = k_at;
+            for (int b = 0; b < g.bits; ++b) out_bit[g.pos + b] = lo_of[l] + k_at + b;
+            k_at += g.bits;
+        }
+        for (int b = 0; b < lg_p[l]; ++b) out_bit[lo_of[l] + b] = lo_of[l] + k_at + b;
+    }
+    if (!contiguous)
+        for (int b = 0; b < a.lg_tile; ++b)
+            if (out_bit[b] >= lg_v) out_bit[b] += a.lg_inner - lg_v;
+    const Dig &df = dg[order[0]], &dl = dg[order[no - 1]];
+    a.in_bit = contiguous ? df.pos : df.pos - lg_v + a.lg_inner;
+    a.out_bit = out_bit[dl.pos];
+    // the last stage's lanes follow the output: its tile bits in order of their output position
+    int tb[32], nt = 0;
+    for (int b = 0; b < a.lg_tile; ++b)
+        if (b < dl.pos || b >= dl.pos + dl.bits) tb[nt++] = b;
+    for (int i = 1; i < nt; ++i)
+        for (int k = i; k > 0 && out_bit[tb[k - 1]] > out_bit[tb[k]]; --k) std::swap(tb[k - 1], tb[k]);
+    for (int i = 0; i < nt;) {
+        int j = i + 1;
+        while (j < nt && tb[j] == tb[j - 1] + 1) ++j;
+        if (a.nlast >= kTpFields) return false;
+        a.last[a.nlast++] = {i, (1 << (j - i)) - 1, tb[i]};
+        i = j;
+    }
+    for (int i = 0; i < nt;) {
+        int j = i + 1;
+        while (j < nt && out_bit[tb[j]] == out_bit[tb[j - 1]] + 1) ++j;
+        if (a.nout >= kTpFields) return false;
+        a.out[a.nout++] = {i, (1 << (j - i)) - 1, out_bit[tb[i]]};
+        i = j;
+    }
+    // exponent groups: the tile bits no digit covers
+    for (int b = 0; b < a.lg_tile;) {
+        bool digit = false;
+        for (int i = 0; i < nd; ++i)
+            if (b >= dg[i].pos && b < dg[i].pos + dg[i].bits) digit = true;
+        if (digit) {
+            ++b;
+            continue;
+        }
+        BitField *f = a.ngroup ? &a.group[a.ngroup - 1] : nullptr;
+        if (f && f->sh + ilog2(f->mask + 1) == b) {
+            f->mask = f->mask * 2 + 1;
+        } else {
+            if (a.ngroup >= kTpFields) return false;
+            a.group[a.ngroup++] = {b, 1, a.lg_groups};
+        }
+        ++a.lg_groups;
+        ++b;
+    }
+    // swizzle: the shifts that leave the lanes of one wavefront (16 of 8 bytes, 8 of 16) in distinct slots
+    const int lw = is_double ? 3 : 4, m = (1 << lw) - 1;
+    int best = 1 << 30;
+    for (int s1 = 1; s1 <= 13; ++s1)
+        for (int s2 = s1; s2 <= 13; ++s2) {
+            auto slot = [&](int e) { return (e ^ (e >> s1) ^ (s2 == s1 ? 0 : e >> s2)) & m; };
+            int cost = 0;
+            for (int si = 0; si < no; ++si) {
+                const Dig &g = dg[order[si]];
+                int v[4], k = 0;
+                if (si == no - 1) {
+                    for (int i = 0; i < lw && i < nt; ++i) v[k++] = slot(1 << tb[i]);
+                } else {
+                    for (int b = 0; b < a.lg_tile && k < lw; ++b)
+                        if (b < g.pos || b >= g.pos + g.bits) v[k++] = slot(1 << b);
+                }
+                cost += (1 << (k - gf2_rank(v, k))) * (si == 0 || si == no - 1 ? 1 : 2);
+            }
+            if (cost < best) {
+                best = cost;
+                a.swz[0] = s1;
+                a.swz[1] = s2 == s1 ? 30 : s2;
+            }
+        }
+    auto slot = [&](int e) { return e ^ ((e >> a.swz[0]) & m) ^ ((e >> a.swz[1]) & m); };
+    int tab = 0;
+    for (int si = 0; si < no; ++si) {
+        const int id = order[si];
+        const Dig &g = dg[id];
+        const int l = g.axis, first = first_of[l], at = id - first;
+        TileStage &s = a.st[si];
+        s.lg_r = g.bits;
+        s.pos = g.pos;
+        s.tw = tw[l];
+        s.tw64 = tw64[l];
+        for (int r = 0; r < 1 << g.bits; ++r) s.rx[r] = slot(r << g.pos);
+        const int lo_m = lo_of[l] + lg_p[l];  // lowest bit of m
+        if (at + 1 < count_of[l]) {  // w_{R T}^{r j} = w_n^{r j n / (R T)}
+            s.tw_kind = 1;
+            s.lo = lo_m;
+            s.lg_q = g.pos - lo_m;
+            s.lg_step = ilog2(n[l]) - g.bits - s.lg_q;
+        } else if (lg_p[l] > 0) {  // w_n^{k s}, k = k_prev + r 2^k_bit
+            s.tw_kind = 2;
+            s.lo = lo_of[l];
+            s.lg_p = lg_p[l];
+            s.lg_q = ilog2(n[l]) - g.bits;
+            s.lg_step = k_bit[id];
+            for (int i = 0; i < at; ++i) {
+                if (s.nk >= 2) return false;
+                const Dig &h = dg[first + i];
+                s.k[s.nk++] = {h.pos - (g.pos + g.bits), (1 << h.bits) - 1, k_bit[first + i]};
+            }
+        }
+        s.tab = tab;
+        if (s.tw_kind) tab += 1 << (g.bits + s.lg_q);
+    }
+    const size_t es = is_double ? 16 : 8;
+    a.tab_off = no > 1 ? es << a.lg_tile : 0;
+    a.emax_off = a.tab_off + tab * es;
+    a.smem = a.emax_off + (is_double ? sizeof(int) << a.lg_groups : 0);
+    // complex128: one fiber of the first stage per thread (its exponent covers all of them); complex64: 16 values
+    a.threads = is_double ? 1 << (a.lg_tile - a.st[0].lg_r) : a.lg_tile > 9 + wide ? 1 << (a.lg_tile - 4 - wide) : 32;
+    if (a.threads > (wide ? 256 : 512) || a.smem > (size_t)kMaxDynSmem) return false;
+    a.scale = 1.0;
+    return true;
+}
+
+cudaError_t prepare_tile_pass(TilePass &a, int is_double, int dir) {
+    if (is_double) return dir < 0 ? prepare_t<kTpFixed, -1>(a) : prepare_t<kTpFixed, 1>(a);
+    if (a.wide) return dir < 0 ? prepare_t<kTpF32w, -1>(a) : prepare_t<kTpF32w, 1>(a);
+    return dir < 0 ? prepare_t<kTpF32, -1>(a) : prepare_t<kTpF32, 1>(a);
+}
+
+cudaError_t launch_tile_pass(const TilePass &a, int is_double, int dir, cudaStream_t st) {
+    if (is_double) return dir < 0 ? launch_t<kTpFixed, -1>(a, st) : launch_t<kTpFixed, 1>(a, st);
+    if (a.wide) return dir < 0 ? launch_t<kTpF32w, -1>(a, st) : launch_t<kTpF32w, 1>(a, st);
+    return dir < 0 ? launch_t<kTpF32, -1>(a, st) : launch_t<kTpF32, 1>(a, st);
+}
+
+}  // namespace fftu

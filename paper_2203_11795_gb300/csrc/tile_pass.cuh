@@ -1,0 +1,259 @@
+// Tile passes: one or more adjacent axes in one HBM round trip, all their positions in a tile.
+//
+// Two forms.  Phase A (Superstep 0 and the Put of Algorithm 2.3, Sec. 2.2): on each axis F_{n_l/p_l} on every residue
+// class s, the twiddle w_{n_l}^{k s}, and the position s n_l/p_l + k.  Whole axes: where the library chooses the grid,
+// fftu_exec needs only the transform and not the data between the supersteps.  Superstep 0, the Put and Superstep 2
+// act on each axis by itself (tensor products, Sec. 2.2), so an axis whose length fits a tile runs all three inside
+// shared memory, as the radix split (Sec. 2.1.1, eq. radix) of one F_{n_l}: phase A and phase B of that axis cost one
+// pass instead of two.
+//
+// The array is viewed as [outer][G][inner] with G the product of the pass' axes.  A tile holds all G positions for
+// V = 2^lg_v adjacent inner positions (inner > 1) or V adjacent outer positions (inner = 1, contiguous memory).
+// Tile index e: [g][v] or [v][g], g row-major over the axes, so tile order is memory order.  Each axis is split
+// into digits of at most 5 bits, highest first; a stage transforms one digit in place:
+//   x[j + T r] (j in [T]: the axis' lower digits) -> F_R over r -> k in the digit's place, times w_{R T}^{k j}.
+// In phase A the digits split m (i = s + p m) and s, the lowest bits of the axis, stays in place until the store.
+// The first stage loads its fibers from HBM into registers and the last one stores them to HBM, with the digits
+// of each axis in reverse (k = k_1 + R_1 k_2 + ...); between stages the tile is in shared memory, one barrier per
+// stage (a stage writes the slots it read).  Every load of a tile precedes its stores, so a pass may be in place.
+//
+// Shared slot of e: e ^ ((e >> swz[0]) & m) ^ ((e >> swz[1]) & m), m = 15 (8-byte elements) or 7 (16-byte): linear over
+// XOR, so the slots of a fiber are the first one's XOR stage constants; the planner picks the shifts that leave
+// the stages' accesses without bank conflicts.
+//
+// Arithmetic: FP32 (complex64); for complex128 fixed point (fixed64.cuh) with one exponent per sub-DFT, and a tile with
+// values that cannot be scaled is run again in FP64 from its input.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "fft_device.cuh"
+#include "fftu_internal.h"
+#include "fixed64.cuh"
+
+namespace fftu {
+
+// ARITH of a tile pass; kTpF32w: complex64 with radix-32 stages (a kernel of its own, with twice the registers)
+constexpr int kTpF32 = 0, kTpFixed = 1, kTpF64 = 2, kTpF32w = 3;
+template <int ARITH> struct tp_type;
+template <> struct tp_type<kTpF32> { using elem = float2; using work = float2; using tw = float2; };
+template <> struct tp_type<kTpF32w> : tp_type<kTpF32> {};
+template <> struct tp_type<kTpFixed> { using elem = double2; using work = longlong2; using tw = int4; };
+template <> struct tp_type<kTpF64> { using elem = double2; using work = double2; using tw = double2; };
+
+template <int ARITH> __device__ __forceinline__ int tp_slot(const TilePass &a, int e) {
+    constexpr int m = sizeof(typename tp_type<ARITH>::elem) == 8 ? 15 : 7;
+    return e ^ ((e >> a.swz[0]) & m) ^ ((e >> a.swz[1]) & m);
+}
+// Not unrolled: the fields (kernel parameters) would otherwise be kept in registers across a CTA's tiles.
+__device__ __forceinline__ unsigned tp_fields(const BitField *f, int n, unsigned x) {
+    unsigned o = 0;
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) o |= ((x >> f[i].sh) & f[i].mask) << f[i].dst;
+    return o;
+}
+
+template <int ARITH, int DIR>
+__device__ __forceinline__ typename tp_type<ARITH>::work tp_twiddle(typename tp_type<ARITH>::work x,
+                                                                    typename tp_type<ARITH>::tw w) {
+    if constexpr (ARITH == kTpFixed) return fx_cmul<DIR>(x, w);
+    else return cmul(x, dirw<DIR>(w));
+}
+template <int ARITH, int DIR, int R> __device__ __forceinline__ void tp_dft(typename tp_type<ARITH>::work *v) {
+    if constexpr (ARITH == kTpFixed) fx_dft<R, DIR>(v);
+    else dft_small<R, DIR>(v);
+}
+
+// The column of stage s's twiddle table for the fiber at tile index e0.
+__device__ __forceinline__ int tp_column(const TileStage &s, int e0) {
+    const int low = (e0 >> s.lo) & ((1 << (s.tw_kind == 1 ? s.lg_q : s.lg_p)) - 1);
+    if (s.tw_kind == 1) return low;
+    const int up = (e0 >> (s.pos + s.lg_r)) & ((1 << (s.lg_q - s.lg_p)) - 1);
+    return low | (up << s.lg_p);
+}
+// Exponent of w_n for output digit r in column q.
+__device__ __forceinline__ unsigned tp_exponent(const TileStage &s, unsigned r, unsigned q) {
+    if (s.tw_kind == 1) return (r * q) << s.lg_step;
+    const unsigned kp = tp_fields(s.k, s.nk, q >> s.lg_p);
+    return (kp + (r << s.lg_step)) * (q & ((1u << s.lg_p) - 1));
+}
+// The twiddles of a stage on its fiber.
+template <int ARITH, int DIR, int R>
+__device__ __forceinline__ void tp_twiddles(const TileStage &s, int e0, typename tp_type<ARITH>::work *v,
+                                            const typename tp_type<ARITH>::tw *tabs) {
+    const int q = tp_column(s, e0);
+    if constexpr (ARITH == kTpF64) {
+        const double2 *tw = static_cast<const double2 *>(s.tw64);
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = cmul(v[r], dirw<DIR>(tw[tp_exponent(s, r, q)]));
+    } else {
+        const typename tp_type<ARITH>::tw *t = tabs + s.tab + q;
+        if (s.tw_kind == 2) v[0] = tp_twiddle<ARITH, DIR>(v[0], t[0]);
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[r] = tp_twiddle<ARITH, DIR>(v[r], t[r << s.lg_q]);
+    }
+}
+
+// One stage of radix R.  FIRST: from src; LAST: to dst (both: a pass of one digit).  Returns false (kTpFixed, FIRST)
+// when the tile needs FP64 arithmetic.  `key` table: one magnitude key per v (kTpFixed).
+template <int ARITH, int DIR, bool MUL, int R, bool FIRST, bool LAST>
+__device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_type<ARITH>::work *sm,
+                                         const typename tp_type<ARITH>::tw *tabs, int *emax,
+                                         const typename tp_type<ARITH>::elem *__restrict__ src,
+                                         typename tp_type<ARITH>::elem *__restrict__ dst) {
+    using T = tp_type<ARITH>;
+    using W = typename T::work;
+    constexpr int RHO = lg_of<R>();
+    int phi0 = threadIdx.x;
+    asm volatile("" : "+r"(si), "+r"(phi0));  // per tile: nothing derived from them is kept in registers across tiles
+    const TileStage &s = a.st[si];
+    const int fibers = 1 << (a.lg_tile - RHO);
+#pragma unroll 1
+    for (int phi = phi0; phi < fibers; phi += blockDim.x) {
+        int e0;
+        if constexpr (LAST && !FIRST) e0 = (int)tp_fields(a.last, a.nlast, (unsigned)phi);
+        else e0 = ((phi >> s.pos) << (s.pos + RHO)) | (phi & ((1 << s.pos) - 1));
+        W v[R];
+        int slot = 0;
+        if constexpr (!(FIRST && LAST)) slot = tp_slot<ARITH>(a, e0);
+        int key = 0;
+        if constexpr (FIRST) {
+            const unsigned off = a.lg_inner < 0 ? (unsigned)e0
+                                                : (((unsigned)e0 >> a.lg_v) << a.lg_inner) | (e0 & ((1 << a.lg_v) - 1));
+            const typename T::elem *p = src + off;
+            if constexpr (ARITH == kTpFixed) {
+                double2 x[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) x[r] = p[(size_t)r << a.in_bit];
+                unsigned lo = 0;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int k = fx_key(x[r]);
+                    key = k > key ? k : key;
+                }
+                if (key == 0) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+                        lo |= (unsigned)__double2loint(x[r].x) | (unsigned)__double2loint(x[r].y);
+                }
+                const int bad = !fx_plain(key, lo);
+                int *em = emax + tp_fields(a.group, a.ngroup, (unsigned)e0);
+                atomicMax(em, key);
+                if (__syncthreads_or(bad)) return false;  // one fiber per thread: every thread is here
+                key = *em;
+                const int E = fx_exp(key);
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    v[r] = mk<longlong2>(fx_in<60 - RHO>(x[r].x, E), fx_in<60 - RHO>(x[r].y, E));
+            } else {
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[r] = p[(size_t)r << a.in_bit];
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                v[r] = sm[slot ^ s.rx[r]];
+                if constexpr (ARITH == kTpFixed) v[r] = fx_scale_down<RHO>(v[r]);
+            }
+        }
+        tp_dft<ARITH, DIR, R>(v);
+        if constexpr (LAST) {
+            if (s.tw_kind) tp_twiddles<ARITH, DIR, R>(s, e0, v, tabs);  // phase A: w_n^{k s} of the last axis
+            typename T::elem *q;
+            if constexpr (FIRST) {
+                const unsigned off = a.lg_inner < 0 ? (unsigned)e0
+                                                    : (((unsigned)e0 >> a.lg_v) << a.lg_inner) | (e0 & ((1 << a.lg_v) - 1));
+                q = dst + off;
+            } else {
+                q = dst + tp_fields(a.out, a.nout, (unsigned)phi);
+            }
+            if constexpr (ARITH == kTpFixed && !FIRST) key = emax[tp_fields(a.group, a.ngroup, (unsigned)e0)];
+            [[maybe_unused]] const int x0 = fx_exp(key) + 3 + a.lg_dft + a.lg_scale;
+            [[maybe_unused]] const auto f = (typename real_of<W>::type)a.scale;
+            // MUL: the pointwise factor at the same natural index
+            [[maybe_unused]] const typename T::elem *m =
+                MUL ? static_cast<const typename T::elem *>(a.mul) + (q - static_cast<typename T::elem *>(a.dst)) : nullptr;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                typename T::elem y;
+                if constexpr (ARITH == kTpFixed) {
+                    if (key == 0) v[r] = mk<longlong2>(0, 0);  // no trace of the products' rounding constants
+                    y = mk<double2>(fx_out(v[r].x, x0), fx_out(v[r].y, x0));
+                } else {
+                    y = a.lg_scale != 0 ? cscale(v[r], f) : v[r];
+                }
+                if constexpr (MUL) y = cmul(y, m[(size_t)r << a.out_bit]);
+                q[(size_t)r << a.out_bit] = y;
+            }
+        } else {
+            if (s.tw_kind) tp_twiddles<ARITH, DIR, R>(s, e0, v, tabs);
+#pragma unroll
+            for (int r = 0; r < R; ++r) sm[slot ^ s.rx[r]] = v[r];
+        }
+    }
+    return true;
+}
+
+template <int ARITH, int DIR, bool MUL, bool FIRST, bool LAST>
+__device__ __forceinline__ bool tp_stage_any(const TilePass &a, int si, typename tp_type<ARITH>::work *sm,
+                                             const typename tp_type<ARITH>::tw *tabs, int *emax,
+                                             const typename tp_type<ARITH>::elem *src,
+                                             typename tp_type<ARITH>::elem *dst) {
+    switch (a.st[si].lg_r) {
+        case 1: return tp_stage<ARITH, DIR, MUL, 2, FIRST, LAST>(a, si, sm, tabs, emax, src, dst);
+        case 2: return tp_stage<ARITH, DIR, MUL, 4, FIRST, LAST>(a, si, sm, tabs, emax, src, dst);
+        case 3: return tp_stage<ARITH, DIR, MUL, 8, FIRST, LAST>(a, si, sm, tabs, emax, src, dst);
+        case 4:
+            if constexpr (ARITH == kTpF32 || ARITH == kTpF32w)
+                return tp_stage<ARITH, DIR, MUL, 16, FIRST, LAST>(a, si, sm, tabs, emax, src, dst);
+            break;
+        default:
+            if constexpr (ARITH == kTpF32w)
+                return tp_stage<ARITH, DIR, MUL, 32, FIRST, LAST>(a, si, sm, tabs, emax, src, dst);
+            break;
+    }
+    return true;
+}
+
+// Twiddle tables of the stages (F32 / Fixed).
+template <int ARITH>
+__device__ __forceinline__ void tp_tables(const TilePass &a, typename tp_type<ARITH>::tw *tabs) {
+    using TW = typename tp_type<ARITH>::tw;
+    for (int si = 0; si < a.nst; ++si) {
+        const TileStage &s = a.st[si];
+        if (s.tw_kind == 0) continue;
+        const TW *tw = static_cast<const TW *>(s.tw);
+        const int n = 1 << (s.lg_r + s.lg_q);
+        for (int i = threadIdx.x; i < n; i += blockDim.x)
+            tabs[s.tab + i] = tw[tp_exponent(s, (unsigned)i >> s.lg_q, (unsigned)i & ((1u << s.lg_q) - 1))];
+    }
+}
+
+template <int ARITH, int DIR, bool MUL>
+__device__ __forceinline__ bool tp_run(const TilePass &a, typename tp_type<ARITH>::work *sm,
+                                       const typename tp_type<ARITH>::tw *tabs, int *emax,
+                                       const typename tp_type<ARITH>::elem *src, typename tp_type<ARITH>::elem *dst) {
+    if (a.nst == 1) return tp_stage_any<ARITH, DIR, MUL, true, true>(a, 0, sm, tabs, emax, src, dst);
+    if (!tp_stage_any<ARITH, DIR, MUL, true, false>(a, 0, sm, tabs, emax, src, dst)) return false;
+    __syncthreads();
+    for (int si = 1; si + 1 < a.nst; ++si) {
+        tp_stage_any<ARITH, DIR, MUL, false, false>(a, si, sm, tabs, emax, src, dst);
+        __syncthreads();
+    }
+    tp_stage_any<ARITH, DIR, MUL, false, true>(a, a.nst - 1, sm, tabs, emax, src, dst);
+    return true;
+}
+
+template <int DIR, bool MUL>
+__device__ __noinline__ void tp_run_fp64(const TilePass &a, double2 *sm, const double2 *src, double2 *dst) {
+    tp_run<kTpF64, DIR, MUL>(a, sm, nullptr, nullptr, src, dst);
+}
+
+// Element offset of tile t.
+__device__ __forceinline__ int64_t tp_base(const TilePass &a, int64_t t) {
+    if (a.lg_inner < 0) return t << a.lg_tile;
+    const int lg_c = a.lg_inner - a.lg_v;  // tiles along the inner positions
+    return ((t >> lg_c) << (a.lg_g + a.lg_inner)) + ((t & (((int64_t)1 << lg_c) - 1)) << a.lg_v);
+}
+
+}  // namespace fftu

@@ -170,6 +170,7 @@ bool autotune(int d, const int64_t *n, fftu_dtype dtype, fftu_dir dir, const fft
 
     fftu_options cur = base;
     cur.tune = 0;
+    const fftu_options base_untuned = cur;
     std::vector<int64_t> best_p;
     float best = -1.f;
     // 1. the grid: q on every axis, and q with the last (contiguous) axis at q / 2
@@ -222,6 +223,17 @@ bool autotune(int d, const int64_t *n, fftu_dtype dtype, fftu_dir dir, const fft
         else try_field(&cur.tile, {2048, 8192});
     }
     if (base.radix == 0 && base.precision == FFTU_PREC_NATIVE) try_field(&cur.radix, {16});
+    // 5. the default grid left to the library (whole-axis passes where they apply), written as schedule AUTO; a choice
+    // measured on a grid of its own is written FUSED where that is what AUTO ran
+    if (base.schedule == FFTU_SCHED_AUTO && base.precision == FFTU_PREC_NATIVE) {
+        const float ms = time_candidate(d, n, nullptr, dtype, dir, base_untuned, in, out);
+        if (ms >= 0.f && ms < best) {
+            for (int l = 0; l < d; ++l) best_p[l] = pmax[l] < 8 ? pmax[l] : 8;
+            cur = base_untuned;
+        } else if (cur.schedule == FFTU_SCHED_AUTO) {
+            cur.schedule = FFTU_SCHED_FUSED;
+        }
+    }
     cudaFree(in);
     cudaFree(out);
     for (int l = 0; l < d; ++l) t->p[l] = best_p[l];
