@@ -436,8 +436,9 @@ bool make_triple_pass(const Plan &pl, TriplePass &a) {
 // 2048 complex128 elements, up to 64 KB.  Runs on a strided group: complex64 16 elements (128 bytes), 8 where 16 do
 // not fit the tile; complex128 4.  Measured on 512 x 512 x 256 complex64 (floor 158 us a pass): the 512-point axes 214 and
 // 358 us at 8, 192 and 190 us at 16; a 1024-point axis 223-279 us at 8, 246-262 us at 16 with a 128 KB tile.
+// batched: for a launch that many transforms share (usual tiles whatever N, no radix-32 stages, at most 256 threads).
 bool choose_tile_pass(int d, const int64_t *n, const int64_t *p, int l1, int l_min, int is_double,
-                      const void *const *tw, const void *const *tw64, int *l0_out, TilePass &a) {
+                      const void *const *tw, const void *const *tw64, bool batched, int *l0_out, TilePass &a) {
     const int target = is_double ? 11 : 12, max_tile = is_double ? 12 : 13, min_v = is_double ? 2 : 3;
     int64_t inner = 1, N = 1;
     for (int l = 0; l < d; ++l) N *= n[l];
@@ -459,14 +460,18 @@ bool choose_tile_pass(int d, const int64_t *n, const int64_t *p, int l1, int l_m
         if (!contiguous && !is_double && lg_v == 3 && lg_g + 4 <= max_tile) lg_v = 4;
         lg_v = std::min(lg_v, contiguous ? ilog2(outer) : lg_in);
         // small arrays: smaller tiles while the GPU is not full
-        while (lg_v > (contiguous ? 0 : need_v) && lg_v + lg_g > 9 && (N >> (lg_g + lg_v)) < 304) --lg_v;
-        if (make_tile_pass(d, n, p, l0, l1, is_double, 0, lg_v, tw, tw64, a)) {
+        while (!batched && lg_v > (contiguous ? 0 : need_v) && lg_v + lg_g > 9 && (N >> (lg_g + lg_v)) < 304) --lg_v;
+        bool ok = make_tile_pass(d, n, p, l0, l1, is_double, 0, lg_v, tw, tw64, a);
+        while (batched && is_double && lg_v > 0 && !(ok && a.threads <= 256))
+            ok = make_tile_pass(d, n, p, l0, l1, is_double, 0, --lg_v, tw, tw64, a);
+        if (batched && is_double && a.threads > 256) ok = false;
+        if (ok) {
             // complex64: radix-32 stages where they save stages (1024-point contiguous lines 210 -> 172 us, strided
             // 259 -> 223 us per 64 M elements).  Not on contiguous groups of several axes (32 x 32 planes: 3 stages 143
             // us against 4 at 132), on single-stage contiguous lines (a thread per line scatters its accesses), or
             // where 32 values a thread leave SMs idle (1024 x 1024: 18 against 11 us).
             TilePass w;
-            if (!is_double && (N >> 22) > 0 && !(contiguous && l0 < l1) &&
+            if (!is_double && !batched && (N >> 22) > 0 && !(contiguous && l0 < l1) &&
                 make_tile_pass(d, n, p, l0, l1, 0, 1, lg_v, tw, tw64, w) && w.nst < a.nst && (w.nst > 1 || !contiguous))
                 a = w;
             *l0_out = l0;
@@ -522,7 +527,7 @@ fftu_status build_generic_phase_a(Plan &pl, std::vector<Step> &out, bool allow_l
                    !(allow_line && l_min > 1 && pl.n[l_min - 1] > 1 && pl.n[l_min - 2] > 1 &&
                      make_pair_pass(pl, l_min - 1, s.pair)))
                 --l_min;
-            if (choose_tile_pass(pl.d, pl.n, pl.p, l, l_min, is_double, tw, tw64, &l0, s.tile)) {
+            if (choose_tile_pass(pl.d, pl.n, pl.p, l, l_min, is_double, tw, tw64, false, &l0, s.tile)) {
                 cudaError_t e = prepare_tile_pass(s.tile, is_double, pl.dir);
                 if (e != cudaSuccess) return cuda_fail(e, "tile pass attributes");
                 s.kind = STEP_TILE;
@@ -588,9 +593,9 @@ fftu_status build_fused_phase_a(Plan &pl, bool *used) {
     return FFTU_OK;
 }
 
-// The whole transform as passes over groups of whole axes (tile_pass.cuh), last axes first; no workspace.  Left
-// empty when some axis does not fit a tile.
-fftu_status build_whole(Plan &pl) {
+// The whole transform as passes over groups of whole axes (tile_pass.cuh), last axes first; no workspace.  false, and
+// no passes, when some axis does not fit a tile.
+bool whole_passes(const Plan &pl, bool batched, std::vector<TilePass> &steps) {
     const int is_double = pl.dtype == FFTU_C128;
     int64_t n[FFTU_MAX_DIMS];
     const void *tw[FFTU_MAX_DIMS], *tw64[FFTU_MAX_DIMS];
@@ -602,20 +607,30 @@ fftu_status build_whole(Plan &pl) {
         tw64[d] = is_double ? pl.table(l) : nullptr;
         ++d;
     }
-    if (d == 0) return FFTU_OK;
-    std::vector<TilePass> steps;
+    steps.clear();
     for (int l1 = d - 1; l1 >= 0;) {
         TilePass a;
         int l0 = l1;
-        if (!choose_tile_pass(d, n, nullptr, l1, 0, is_double, tw, tw64, &l0, a)) return FFTU_OK;
-        cudaError_t e = prepare_tile_pass(a, is_double, pl.dir);
-        if (e != cudaSuccess) return cuda_fail(e, "tile pass attributes");
+        if (!choose_tile_pass(d, n, nullptr, l1, 0, is_double, tw, tw64, batched, &l0, a)) {
+            steps.clear();
+            return false;
+        }
         steps.push_back(a);
         l1 = l0 - 1;
     }
-    if (pl.dir == FFTU_INVERSE) {
+    if (pl.dir == FFTU_INVERSE && !steps.empty()) {
         steps.back().scale = 1.0 / (double)pl.N;
         steps.back().lg_scale = -ilog2(pl.N);
+    }
+    return !steps.empty();
+}
+
+fftu_status build_whole(Plan &pl) {
+    std::vector<TilePass> steps;
+    if (!whole_passes(pl, false, steps)) return FFTU_OK;
+    for (TilePass &a : steps) {
+        cudaError_t e = prepare_tile_pass(a, pl.dtype == FFTU_C128, pl.dir);
+        if (e != cudaSuccess) return cuda_fail(e, "tile pass attributes");
     }
     pl.whole = steps;
     return FFTU_OK;
@@ -794,6 +809,8 @@ fftu_status plan_view(fftu_handle h, PlanView *v) {
     v->radix = pl.radix;
     v->a_passes.clear();
     v->b_steps.clear();
+    v->whole.clear();
+    if (!pl.whole.empty()) whole_passes(pl, true, v->whole);
     const bool fused_a = !pl.phase_a.empty() && pl.phase_a[0].kind == STEP_PHASE_A3;
     for (const Step &s : fused_a ? pl.phase_a_inplace : pl.phase_a) {
         StepView sv;

@@ -215,6 +215,9 @@ struct PlanView {
     int radix;                      // stage radix of the strided passes (8 or 16)
     std::vector<StepView> a_passes;  // phase A, generic passes (first reads in, then in place on out)
     std::vector<StepView> b_steps;   // phase B, in place on out
+    // the whole transform as tile passes of at most 256 threads (first reads in, then in place on out), where the plan
+    // runs that way; empty otherwise
+    std::vector<TilePass> whole;
 };
 fftu_status plan_view(fftu_handle h, PlanView *v);
 

@@ -13,7 +13,7 @@ namespace {
 
 // Persistent: the twiddle tables are built once per CTA.  Registers: 64 for complex64 (two CTAs of 512 threads, four of
 // 256), 80 for complex128 (the bound of 768 threads; three CTAs of 256).
-template <int ARITH, int DIR, bool MUL>
+template <int ARITH, int DIR, int OPT>
 __global__ void __launch_bounds__(ARITH == kTpF32 ? 512 : ARITH == kTpF32w ? 256 : 768, ARITH == kTpFixed ? 1 : 2) tile_pass_kernel(const __grid_constant__ TilePass a) {
     using T = tp_type<ARITH>;
     using E = typename T::elem;
@@ -21,7 +21,11 @@ __global__ void __launch_bounds__(ARITH == kTpF32 ? 512 : ARITH == kTpF32w ? 256
     auto *sm = reinterpret_cast<typename T::work *>(tp_raw);
     auto *tabs = reinterpret_cast<typename T::tw *>(tp_raw + a.tab_off);
     int *emax = reinterpret_cast<int *>(tp_raw + a.emax_off);
-    tp_tables<ARITH>(a, tabs);
+    // The next kernel of the stream may start once every CTA of this one has; it waits below for all of this kernel's
+    // writes, as this one does for its predecessor's (small arrays are bound by launch and table latency).
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    tp_tables<ARITH>(a, tabs);  // plan data, not written by earlier kernels
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int64_t t = blockIdx.x; t < a.tiles; t += gridDim.x) {
         __syncthreads();  // tables ready; the previous tile's last stage done with its slots and exponents
         if constexpr (ARITH == kTpFixed) {
@@ -31,8 +35,8 @@ __global__ void __launch_bounds__(ARITH == kTpF32 ? 512 : ARITH == kTpF32w ? 256
         const int64_t base = tp_base(a, t);
         const E *src = static_cast<const E *>(a.src) + base;
         E *dst = static_cast<E *>(a.dst) + base;
-        if (!tp_run<ARITH, DIR, MUL>(a, sm, tabs, emax, src, dst)) {
-            if constexpr (ARITH == kTpFixed) tp_run_fp64<DIR, MUL>(a, reinterpret_cast<double2 *>(sm), src, dst);
+        if (!tp_run<ARITH, DIR, OPT>(a, sm, tabs, emax, src, dst)) {
+            if constexpr (ARITH == kTpFixed) tp_run_fp64<DIR, OPT>(a, reinterpret_cast<double2 *>(sm), src, dst);
         }
     }
 }
@@ -79,25 +83,33 @@ int gf2_rank(int *v, int n) {
 template <int ARITH, int DIR>
 cudaError_t launch_t(const TilePass &a, cudaStream_t st) {
     int64_t grid = a.tiles < a.grid ? a.tiles : a.grid;
-    if (a.mul)
-        tile_pass_kernel<ARITH, DIR, true><<<(unsigned)grid, a.threads, a.smem, st>>>(a);
-    else
-        tile_pass_kernel<ARITH, DIR, false><<<(unsigned)grid, a.threads, a.smem, st>>>(a);
-    return cudaGetLastError();
+    // programmatic launch: the CTAs may start, and build their tables, while the kernel before this one finishes
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)a.threads);
+    cfg.dynamicSmemBytes = a.smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return a.mul ? cudaLaunchKernelEx(&cfg, tile_pass_kernel<ARITH, DIR, kTpMul>, a)
+                 : cudaLaunchKernelEx(&cfg, tile_pass_kernel<ARITH, DIR, 0>, a);
 }
 
 template <int ARITH, int DIR>
 cudaError_t prepare_t(TilePass &a) {
-    cudaError_t e = cudaFuncSetAttribute(tile_pass_kernel<ARITH, DIR, false>,
+    cudaError_t e = cudaFuncSetAttribute(tile_pass_kernel<ARITH, DIR, 0>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tile_pass_kernel<ARITH, DIR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(tile_pass_kernel<ARITH, DIR, kTpMul>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kMaxDynSmem);
     int dev = 0, sms = 0, per_sm = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tile_pass_kernel<ARITH, DIR, false>, a.threads, a.smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tile_pass_kernel<ARITH, DIR, 0>, a.threads, a.smem);
     if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
     a.grid = sms * per_sm;
     return e;

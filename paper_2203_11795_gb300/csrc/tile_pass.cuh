@@ -35,6 +35,9 @@ namespace fftu {
 
 // ARITH of a tile pass; kTpF32w: complex64 with radix-32 stages (a kernel of its own, with twice the registers)
 constexpr int kTpF32 = 0, kTpFixed = 1, kTpF64 = 2, kTpF32w = 3;
+// OPT bits: the pointwise product in the last store; twiddles straight from the root tables (many kinds of pass in one
+// launch) instead of the stages' shared tables
+constexpr int kTpMul = 1, kTpGlobalTw = 2;
 template <int ARITH> struct tp_type;
 template <> struct tp_type<kTpF32> { using elem = float2; using work = float2; using tw = float2; };
 template <> struct tp_type<kTpF32w> : tp_type<kTpF32> {};
@@ -64,6 +67,12 @@ template <int ARITH, int DIR, int R> __device__ __forceinline__ void tp_dft(type
     else dft_small<R, DIR>(v);
 }
 
+// Load of an input element.  In a launch whose passes follow one another (kTpGlobalTw) other SMs wrote it during the
+// kernel: from L2.
+template <int OPT, typename E> __device__ __forceinline__ E tp_load(const E *p) {
+    if constexpr ((OPT & kTpGlobalTw) != 0) return __ldcg(p);
+    else return *p;
+}
 // The column of stage s's twiddle table for the fiber at tile index e0.
 __device__ __forceinline__ int tp_column(const TileStage &s, int e0) {
     const int low = (e0 >> s.lo) & ((1 << (s.tw_kind == 1 ? s.lg_q : s.lg_p)) - 1);
@@ -78,7 +87,7 @@ __device__ __forceinline__ unsigned tp_exponent(const TileStage &s, unsigned r, 
     return (kp + (r << s.lg_step)) * (q & ((1u << s.lg_p) - 1));
 }
 // The twiddles of a stage on its fiber.
-template <int ARITH, int DIR, int R>
+template <int ARITH, int DIR, int OPT, int R>
 __device__ __forceinline__ void tp_twiddles(const TileStage &s, int e0, typename tp_type<ARITH>::work *v,
                                             const typename tp_type<ARITH>::tw *tabs) {
     const int q = tp_column(s, e0);
@@ -86,6 +95,11 @@ __device__ __forceinline__ void tp_twiddles(const TileStage &s, int e0, typename
         const double2 *tw = static_cast<const double2 *>(s.tw64);
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = cmul(v[r], dirw<DIR>(tw[tp_exponent(s, r, q)]));
+    } else if constexpr ((OPT & kTpGlobalTw) != 0) {
+        const typename tp_type<ARITH>::tw *tw = static_cast<const typename tp_type<ARITH>::tw *>(s.tw);
+        if (s.tw_kind == 2) v[0] = tp_twiddle<ARITH, DIR>(v[0], __ldg(tw + tp_exponent(s, 0, q)));
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[r] = tp_twiddle<ARITH, DIR>(v[r], __ldg(tw + tp_exponent(s, r, q)));
     } else {
         const typename tp_type<ARITH>::tw *t = tabs + s.tab + q;
         if (s.tw_kind == 2) v[0] = tp_twiddle<ARITH, DIR>(v[0], t[0]);
@@ -96,11 +110,11 @@ __device__ __forceinline__ void tp_twiddles(const TileStage &s, int e0, typename
 
 // One stage of radix R.  FIRST: from src; LAST: to dst (both: a pass of one digit).  Returns false (kTpFixed, FIRST)
 // when the tile needs FP64 arithmetic.  `key` table: one magnitude key per v (kTpFixed).
-template <int ARITH, int DIR, bool MUL, int R, bool FIRST, bool LAST>
+template <int ARITH, int DIR, int OPT, int R, bool FIRST, bool LAST>
 __device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_type<ARITH>::work *sm,
                                          const typename tp_type<ARITH>::tw *tabs, int *emax,
-                                         const typename tp_type<ARITH>::elem *__restrict__ src,
-                                         typename tp_type<ARITH>::elem *__restrict__ dst) {
+                                         const typename tp_type<ARITH>::elem *src,
+                                         typename tp_type<ARITH>::elem *dst) {
     using T = tp_type<ARITH>;
     using W = typename T::work;
     constexpr int RHO = lg_of<R>();
@@ -108,8 +122,10 @@ __device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_
     asm volatile("" : "+r"(si), "+r"(phi0));  // per tile: nothing derived from them is kept in registers across tiles
     const TileStage &s = a.st[si];
     const int fibers = 1 << (a.lg_tile - RHO);
+    // kTpFixed, FIRST: one fiber per thread at most (blockDim >= fibers), every thread at the barrier
+    constexpr bool kOnce = ARITH == kTpFixed && FIRST;
 #pragma unroll 1
-    for (int phi = phi0; phi < fibers; phi += blockDim.x) {
+    for (int phi = phi0; kOnce || phi < fibers; phi += blockDim.x) {
         int e0;
         if constexpr (LAST && !FIRST) e0 = (int)tp_fields(a.last, a.nlast, (unsigned)phi);
         else e0 = ((phi >> s.pos) << (s.pos + RHO)) | (phi & ((1 << s.pos) - 1));
@@ -123,8 +139,13 @@ __device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_
             const typename T::elem *p = src + off;
             if constexpr (ARITH == kTpFixed) {
                 double2 x[R];
+                if (phi < fibers) {
 #pragma unroll
-                for (int r = 0; r < R; ++r) x[r] = p[(size_t)r << a.in_bit];
+                    for (int r = 0; r < R; ++r) x[r] = tp_load<OPT>(p + ((size_t)r << a.in_bit));
+                } else {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) x[r] = mk<double2>(0.0, 0.0);
+                }
                 unsigned lo = 0;
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
@@ -138,8 +159,9 @@ __device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_
                 }
                 const int bad = !fx_plain(key, lo);
                 int *em = emax + tp_fields(a.group, a.ngroup, (unsigned)e0);
-                atomicMax(em, key);
-                if (__syncthreads_or(bad)) return false;  // one fiber per thread: every thread is here
+                if (phi < fibers) atomicMax(em, key);
+                if (__syncthreads_or(bad)) return false;
+                if (phi >= fibers) break;
                 key = *em;
                 const int E = fx_exp(key);
 #pragma unroll
@@ -147,7 +169,7 @@ __device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_
                     v[r] = mk<longlong2>(fx_in<60 - RHO>(x[r].x, E), fx_in<60 - RHO>(x[r].y, E));
             } else {
 #pragma unroll
-                for (int r = 0; r < R; ++r) v[r] = p[(size_t)r << a.in_bit];
+                for (int r = 0; r < R; ++r) v[r] = tp_load<OPT>(p + ((size_t)r << a.in_bit));
             }
         } else {
 #pragma unroll
@@ -158,7 +180,7 @@ __device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_
         }
         tp_dft<ARITH, DIR, R>(v);
         if constexpr (LAST) {
-            if (s.tw_kind) tp_twiddles<ARITH, DIR, R>(s, e0, v, tabs);  // phase A: w_n^{k s} of the last axis
+            if (s.tw_kind) tp_twiddles<ARITH, DIR, OPT, R>(s, e0, v, tabs);  // phase A: w_n^{k s} of the last axis
             typename T::elem *q;
             if constexpr (FIRST) {
                 const unsigned off = a.lg_inner < 0 ? (unsigned)e0
@@ -170,9 +192,9 @@ __device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_
             if constexpr (ARITH == kTpFixed && !FIRST) key = emax[tp_fields(a.group, a.ngroup, (unsigned)e0)];
             [[maybe_unused]] const int x0 = fx_exp(key) + 3 + a.lg_dft + a.lg_scale;
             [[maybe_unused]] const auto f = (typename real_of<W>::type)a.scale;
-            // MUL: the pointwise factor at the same natural index
+            // kTpMul: the pointwise factor at the same natural index
             [[maybe_unused]] const typename T::elem *m =
-                MUL ? static_cast<const typename T::elem *>(a.mul) + (q - static_cast<typename T::elem *>(a.dst)) : nullptr;
+                (OPT & kTpMul) ? static_cast<const typename T::elem *>(a.mul) + (q - static_cast<typename T::elem *>(a.dst)) : nullptr;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 typename T::elem y;
@@ -182,34 +204,35 @@ __device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_
                 } else {
                     y = a.lg_scale != 0 ? cscale(v[r], f) : v[r];
                 }
-                if constexpr (MUL) y = cmul(y, m[(size_t)r << a.out_bit]);
+                if constexpr ((OPT & kTpMul) != 0) y = cmul(y, m[(size_t)r << a.out_bit]);
                 q[(size_t)r << a.out_bit] = y;
             }
         } else {
-            if (s.tw_kind) tp_twiddles<ARITH, DIR, R>(s, e0, v, tabs);
+            if (s.tw_kind) tp_twiddles<ARITH, DIR, OPT, R>(s, e0, v, tabs);
 #pragma unroll
             for (int r = 0; r < R; ++r) sm[slot ^ s.rx[r]] = v[r];
         }
+        if constexpr (kOnce) break;
     }
     return true;
 }
 
-template <int ARITH, int DIR, bool MUL, bool FIRST, bool LAST>
+template <int ARITH, int DIR, int OPT, bool FIRST, bool LAST>
 __device__ __forceinline__ bool tp_stage_any(const TilePass &a, int si, typename tp_type<ARITH>::work *sm,
                                              const typename tp_type<ARITH>::tw *tabs, int *emax,
                                              const typename tp_type<ARITH>::elem *src,
                                              typename tp_type<ARITH>::elem *dst) {
     switch (a.st[si].lg_r) {
-        case 1: return tp_stage<ARITH, DIR, MUL, 2, FIRST, LAST>(a, si, sm, tabs, emax, src, dst);
-        case 2: return tp_stage<ARITH, DIR, MUL, 4, FIRST, LAST>(a, si, sm, tabs, emax, src, dst);
-        case 3: return tp_stage<ARITH, DIR, MUL, 8, FIRST, LAST>(a, si, sm, tabs, emax, src, dst);
+        case 1: return tp_stage<ARITH, DIR, OPT, 2, FIRST, LAST>(a, si, sm, tabs, emax, src, dst);
+        case 2: return tp_stage<ARITH, DIR, OPT, 4, FIRST, LAST>(a, si, sm, tabs, emax, src, dst);
+        case 3: return tp_stage<ARITH, DIR, OPT, 8, FIRST, LAST>(a, si, sm, tabs, emax, src, dst);
         case 4:
             if constexpr (ARITH == kTpF32 || ARITH == kTpF32w)
-                return tp_stage<ARITH, DIR, MUL, 16, FIRST, LAST>(a, si, sm, tabs, emax, src, dst);
+                return tp_stage<ARITH, DIR, OPT, 16, FIRST, LAST>(a, si, sm, tabs, emax, src, dst);
             break;
         default:
             if constexpr (ARITH == kTpF32w)
-                return tp_stage<ARITH, DIR, MUL, 32, FIRST, LAST>(a, si, sm, tabs, emax, src, dst);
+                return tp_stage<ARITH, DIR, OPT, 32, FIRST, LAST>(a, si, sm, tabs, emax, src, dst);
             break;
     }
     return true;
@@ -229,24 +252,24 @@ __device__ __forceinline__ void tp_tables(const TilePass &a, typename tp_type<AR
     }
 }
 
-template <int ARITH, int DIR, bool MUL>
+template <int ARITH, int DIR, int OPT>
 __device__ __forceinline__ bool tp_run(const TilePass &a, typename tp_type<ARITH>::work *sm,
                                        const typename tp_type<ARITH>::tw *tabs, int *emax,
                                        const typename tp_type<ARITH>::elem *src, typename tp_type<ARITH>::elem *dst) {
-    if (a.nst == 1) return tp_stage_any<ARITH, DIR, MUL, true, true>(a, 0, sm, tabs, emax, src, dst);
-    if (!tp_stage_any<ARITH, DIR, MUL, true, false>(a, 0, sm, tabs, emax, src, dst)) return false;
+    if (a.nst == 1) return tp_stage_any<ARITH, DIR, OPT, true, true>(a, 0, sm, tabs, emax, src, dst);
+    if (!tp_stage_any<ARITH, DIR, OPT, true, false>(a, 0, sm, tabs, emax, src, dst)) return false;
     __syncthreads();
     for (int si = 1; si + 1 < a.nst; ++si) {
-        tp_stage_any<ARITH, DIR, MUL, false, false>(a, si, sm, tabs, emax, src, dst);
+        tp_stage_any<ARITH, DIR, OPT, false, false>(a, si, sm, tabs, emax, src, dst);
         __syncthreads();
     }
-    tp_stage_any<ARITH, DIR, MUL, false, true>(a, a.nst - 1, sm, tabs, emax, src, dst);
+    tp_stage_any<ARITH, DIR, OPT, false, true>(a, a.nst - 1, sm, tabs, emax, src, dst);
     return true;
 }
 
-template <int DIR, bool MUL>
+template <int DIR, int OPT>
 __device__ __noinline__ void tp_run_fp64(const TilePass &a, double2 *sm, const double2 *src, double2 *dst) {
-    tp_run<kTpF64, DIR, MUL>(a, sm, nullptr, nullptr, src, dst);
+    tp_run<kTpF64, DIR, OPT>(a, sm, nullptr, nullptr, src, dst);
 }
 
 // Element offset of tile t.
