@@ -22,6 +22,7 @@
 #include "fft_device.cuh"
 #include "fftu_internal.h"
 #include "generic_tiles.cuh"
+#include "tile_pass.cuh"
 
 namespace fftu {
 
@@ -141,6 +142,94 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(const __grid_const
     }
 }
 
+// A batch whose transforms all run as whole-axis tile passes: the jobs are those passes (2 or 3 per transform instead of
+// the strided kernel's 3 or 4, each with fewer trips through shared memory).
+struct TileJob {
+    int transform, dep;
+    int64_t first, dep_tiles;
+    TilePass a;
+};
+
+struct TileParams {
+    const TileJob *jobs;
+    const int64_t *firsts;
+    int njobs;
+    int64_t total;
+    unsigned long long *task_ctr;
+    unsigned *done;
+    int *status;
+    long long spin_limit_ns;
+    const void *in[kMaxBatch];
+    void *out[kMaxBatch];
+};
+
+constexpr int kTileBatchThreads = 256;
+
+// The tasks in order with their bounded waits as in batch_kernel.  Twiddles come straight from the root tables (a CTA's
+// next tile is usually another job's).  Four CTAs per SM for complex64 (64 registers), three for complex128 (80).
+template <int ARITH, int DIR>
+__global__ void __launch_bounds__(kTileBatchThreads, ARITH == kTpF32 ? 4 : 3)
+    tile_batch_kernel(const __grid_constant__ TileParams P, int emax_off) {
+    using T = tp_type<ARITH>;
+    using E = typename T::elem;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    auto *sm = reinterpret_cast<typename T::work *>(smem_raw);
+    int *emax = reinterpret_cast<int *>(smem_raw + emax_off);
+    __shared__ __align__(16) TileJob s_job;
+    __shared__ long long s_task;
+    __shared__ int s_jobi, s_ok, s_loaded;
+    const int tid = threadIdx.x;
+    if (tid == 0) s_loaded = -1;
+    __syncthreads();
+    for (;;) {
+        if (tid == 0) {
+            const long long t = (long long)atomicAdd(P.task_ctr, 1ull);
+            s_task = t;
+            if (t < P.total) {
+                int lo = 0, hi = P.njobs - 1;  // last job with first <= t
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (__ldg(P.firsts + mid) <= t) lo = mid;
+                    else hi = mid - 1;
+                }
+                s_jobi = lo;
+            }
+        }
+        __syncthreads();
+        const long long t = s_task;
+        if (t >= P.total) break;
+        const int j = s_jobi;
+        if (j != s_loaded) {
+            const int *srcw = reinterpret_cast<const int *>(P.jobs + j);
+            int *dstw = reinterpret_cast<int *>(&s_job);
+            for (int w = tid; w < (int)(sizeof(TileJob) / sizeof(int)); w += blockDim.x) dstw[w] = srcw[w];
+        }
+        __syncthreads();
+        const TilePass &a = s_job.a;
+        if (tid == 0) {
+            s_loaded = j;
+            const int dep = s_job.dep;
+            s_ok = dep < 0 || wait_counter_geq(P.done + dep, (unsigned)s_job.dep_tiles, P.spin_limit_ns, P.status);
+        }
+        if constexpr (ARITH == kTpFixed)
+            for (int i = tid; i < 1 << a.lg_groups; i += blockDim.x) emax[i] = 0;
+        __syncthreads();
+        if (s_ok) {
+            const int64_t base = tp_base(a, t - s_job.first);
+            E *out = static_cast<E *>(P.out[s_job.transform]) + base;
+            const E *src = s_job.dep < 0 ? static_cast<const E *>(P.in[s_job.transform]) + base : out;
+            if (!tp_run<ARITH, DIR, kTpGlobalTw>(a, sm, nullptr, emax, src, out)) {
+                if constexpr (ARITH == kTpFixed) tp_run_fp64<DIR, kTpGlobalTw>(a, reinterpret_cast<double2 *>(sm), src, out);
+            }
+        }
+        __syncthreads();
+        if (tid == 0) {
+            __threadfence();
+            atomicAdd(P.done + j, 1u);
+        }
+    }
+}
+
 // Diagnostic for fftu_selftest_bounded_wait: one thread waits, with the batch kernel's bounded
 // wait, on words[0], which nothing advances; the expired wait leaves FFTU_ERR_TIMEOUT in words[1]
 // and the time it waited in words[2..3].
@@ -170,6 +259,21 @@ cudaError_t batch_setup(size_t smem, int threads, int *grid) {
     return cudaSuccess;
 }
 
+template <int ARITH, int DIR>
+cudaError_t tile_batch_setup(size_t smem, int *grid) {
+    if (smem > (size_t)kMaxDynSmem) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(tile_batch_kernel<ARITH, DIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kMaxDynSmem);
+    int dev = 0, sms = 0, per_sm = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tile_batch_kernel<ARITH, DIR>, kTileBatchThreads, smem);
+    if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
+    *grid = sms * per_sm;
+    return e;
+}
+
 }  // namespace
 
 struct Batch {
@@ -180,6 +284,8 @@ struct Batch {
     int64_t total = 0;
     void *dev_mem = nullptr;  // jobs | firsts | task counter | done counters
     BatchJob *jobs = nullptr;
+    TileJob *tile_jobs = nullptr;  // set instead of jobs when every transform runs as tile passes
+    int emax_off = 0;
     int64_t *firsts = nullptr;
     unsigned long long *task_ctr = nullptr;
     unsigned *done = nullptr;
@@ -214,7 +320,30 @@ fftu_status batch_create(int count, const fftu_handle *plans, Batch **out_batch)
             return FFTU_ERR_UNSUPPORTED;
         }
     }
+    bool tiles = true;
+    for (auto &v : views) tiles = tiles && !v.whole.empty();
     // jobs, pass-major
+    std::vector<TileJob> tjobs;
+    size_t tile_elems = 0, groups = 0;
+    if (tiles) {
+        std::vector<int> last(count, -1);
+        size_t most = 0;
+        for (auto &v : views) most = std::max(most, v.whole.size());
+        for (size_t k = 0; k < most; ++k)
+            for (int i = 0; i < count; ++i) {
+                if (k >= views[i].whole.size()) continue;
+                TileJob J;
+                std::memset(&J, 0, sizeof(J));
+                J.transform = i;
+                J.a = views[i].whole[k];
+                J.dep = last[i];
+                J.dep_tiles = last[i] < 0 ? 0 : tjobs[last[i]].a.tiles;
+                last[i] = (int)tjobs.size();
+                tjobs.push_back(J);
+                tile_elems = std::max(tile_elems, (size_t)1 << J.a.lg_tile);
+                groups = std::max(groups, (size_t)1 << J.a.lg_groups);
+            }
+    }
     std::vector<BatchJob> jobs;
     std::vector<std::vector<int>> job_of(count);
     size_t max_tile_bytes = 0;
@@ -222,7 +351,7 @@ fftu_status batch_create(int count, const fftu_handle *plans, Batch **out_batch)
     int max_passes = 0;
     int max_threads = 128;  // phase-B tiles loop over any block size
     for (auto &v : views) max_passes = std::max(max_passes, (int)(v.a_passes.size() + v.b_steps.size()));
-    for (int k = 0; k < max_passes; ++k) {
+    for (int k = 0; k < (tiles ? 0 : max_passes); ++k) {
         for (int i = 0; i < count; ++i) {
             const PlanView &v = views[i];
             const int na = (int)v.a_passes.size();
@@ -252,7 +381,8 @@ fftu_status batch_create(int count, const fftu_handle *plans, Batch **out_batch)
             jobs.push_back(J);
         }
     }
-    if ((int)jobs.size() > kMaxBatchJobs) {
+    const size_t njobs = tiles ? tjobs.size() : jobs.size();
+    if (njobs > (size_t)kMaxBatchJobs) {
         record_error("batch: too many passes in total");
         return FFTU_ERR_UNSUPPORTED;
     }
@@ -263,11 +393,11 @@ fftu_status batch_create(int count, const fftu_handle *plans, Batch **out_batch)
             return FFTU_ERR_UNSUPPORTED;
         }
     int64_t first = 0;
-    std::vector<int64_t> firsts(jobs.size());
-    for (size_t j = 0; j < jobs.size(); ++j) {
-        jobs[j].first = first;
+    std::vector<int64_t> firsts(njobs);
+    for (size_t j = 0; j < njobs; ++j) {
+        (tiles ? tjobs[j].first : jobs[j].first) = first;
         firsts[j] = first;
-        first += jobs[j].tiles;
+        first += tiles ? tjobs[j].a.tiles : jobs[j].tiles;
     }
     Batch *b = new (std::nothrow) Batch();
     if (!b) {
@@ -278,12 +408,13 @@ fftu_status batch_create(int count, const fftu_handle *plans, Batch **out_batch)
     b->is_double = views[0].dtype == FFTU_C128;
     b->dir = views[0].dir;
     b->device = views[0].device;
-    b->njobs = (int)jobs.size();
+    b->njobs = (int)njobs;
     b->total = first;
-    b->smem = max_tile_bytes;
-    b->threads = std::min(kBatchThreads, (max_threads + 31) / 32 * 32);
-    const size_t jb = sizeof(BatchJob) * jobs.size(), fb = sizeof(int64_t) * jobs.size();
-    b->counter_bytes = 16 + sizeof(unsigned) * jobs.size();
+    b->emax_off = (int)(tile_elems * esize);
+    b->smem = tiles ? tile_elems * esize + (b->is_double ? groups * sizeof(int) : 0) : max_tile_bytes;
+    b->threads = tiles ? kTileBatchThreads : std::min(kBatchThreads, (max_threads + 31) / 32 * 32);
+    const size_t jb = (tiles ? sizeof(TileJob) : sizeof(BatchJob)) * njobs, fb = sizeof(int64_t) * njobs;
+    b->counter_bytes = 16 + sizeof(unsigned) * njobs;
     const size_t bytes = jb + fb + b->counter_bytes + 16;
     cudaError_t e = cudaMalloc(&b->dev_mem, bytes);
     if (e != cudaSuccess) {
@@ -293,7 +424,8 @@ fftu_status batch_create(int count, const fftu_handle *plans, Batch **out_batch)
         return FFTU_ERR_NOMEM;
     }
     char *base = static_cast<char *>(b->dev_mem);
-    b->jobs = reinterpret_cast<BatchJob *>(base);
+    if (tiles) b->tile_jobs = reinterpret_cast<TileJob *>(base);
+    else b->jobs = reinterpret_cast<BatchJob *>(base);
     b->firsts = reinterpret_cast<int64_t *>(base + jb);
     b->task_ctr = reinterpret_cast<unsigned long long *>(base + jb + fb);
     b->status = reinterpret_cast<int *>(base + jb + fb + 8);
@@ -301,12 +433,20 @@ fftu_status batch_create(int count, const fftu_handle *plans, Batch **out_batch)
     // uploads on a private stream: creating a batch does not wait for transforms in flight
     cudaStream_t ps = nullptr;
     e = cudaStreamCreateWithFlags(&ps, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(b->jobs, jobs.data(), jb, cudaMemcpyHostToDevice, ps);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(b->dev_mem, tiles ? (const void *)tjobs.data() : (const void *)jobs.data(), jb,
+                                             cudaMemcpyHostToDevice, ps);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->firsts, firsts.data(), fb, cudaMemcpyHostToDevice, ps);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->status, 0, sizeof(int), ps);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ps);
     if (ps) cudaStreamDestroy(ps);
-    if (e == cudaSuccess) {
+    if (e == cudaSuccess && tiles) {
+        if (b->is_double)
+            e = b->dir < 0 ? tile_batch_setup<kTpFixed, -1>(b->smem, &b->grid)
+                           : tile_batch_setup<kTpFixed, 1>(b->smem, &b->grid);
+        else
+            e = b->dir < 0 ? tile_batch_setup<kTpF32, -1>(b->smem, &b->grid)
+                           : tile_batch_setup<kTpF32, 1>(b->smem, &b->grid);
+    } else if (e == cudaSuccess) {
         if (b->is_double)
             e = b->dir < 0 ? batch_setup<double2, -1>(b->smem, b->threads, &b->grid)
                            : batch_setup<double2, 1>(b->smem, b->threads, &b->grid);
@@ -324,10 +464,10 @@ fftu_status batch_create(int count, const fftu_handle *plans, Batch **out_batch)
     return FFTU_OK;
 }
 
-fftu_status batch_exec(Batch *b, const void *const *ins, void *const *outs, cudaStream_t st) {
-    BatchParams P;
+template <typename PARAMS, typename JOB>
+fftu_status fill_params(Batch *b, const JOB *jobs, const void *const *ins, void *const *outs, PARAMS &P) {
     std::memset(&P, 0, sizeof(P));
-    P.jobs = b->jobs;
+    P.jobs = jobs;
     P.firsts = b->firsts;
     P.njobs = b->njobs;
     P.total = b->total;
@@ -343,6 +483,14 @@ fftu_status batch_exec(Batch *b, const void *const *ins, void *const *outs, cuda
         P.in[i] = ins[i];
         P.out[i] = outs[i];
     }
+    return FFTU_OK;
+}
+
+fftu_status batch_exec(Batch *b, const void *const *ins, void *const *outs, cudaStream_t st) {
+    BatchParams P;
+    TileParams Q;
+    fftu_status s = b->tile_jobs ? fill_params(b, b->tile_jobs, ins, outs, Q) : fill_params(b, b->jobs, ins, outs, P);
+    if (s != FFTU_OK) return s;
     // the task counter and the per-job counters start at zero on every exec
     cudaError_t e = cudaMemsetAsync(b->task_ctr, 0, 8, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->done, 0, sizeof(unsigned) * b->njobs, st);
@@ -352,7 +500,16 @@ fftu_status batch_exec(Batch *b, const void *const *ins, void *const *outs, cuda
     }
     int64_t grid = b->grid;
     if (grid > b->total) grid = b->total;
-    if (b->is_double) {
+    if (b->tile_jobs) {
+        const unsigned g = (unsigned)grid;
+        if (b->is_double) {
+            if (b->dir < 0) tile_batch_kernel<kTpFixed, -1><<<g, b->threads, b->smem, st>>>(Q, b->emax_off);
+            else tile_batch_kernel<kTpFixed, 1><<<g, b->threads, b->smem, st>>>(Q, b->emax_off);
+        } else {
+            if (b->dir < 0) tile_batch_kernel<kTpF32, -1><<<g, b->threads, b->smem, st>>>(Q, b->emax_off);
+            else tile_batch_kernel<kTpF32, 1><<<g, b->threads, b->smem, st>>>(Q, b->emax_off);
+        }
+    } else if (b->is_double) {
         if (b->dir < 0)
             batch_kernel<double2, -1><<<(unsigned)grid, b->threads, b->smem, st>>>(P);
         else

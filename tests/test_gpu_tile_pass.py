@@ -112,3 +112,29 @@ def test_values_out_of_the_fixed_point_range(fftu, kind):
         return
     ref = oracle.fftn(x * s)
     assert oracle.rel_l2(y * s, ref) <= 1e-12 and oracle.rel_l2(z * s, ref) <= 1e-12
+
+
+@pytest.mark.parametrize("dt", [np.complex64, np.complex128])
+@pytest.mark.parametrize("inplace", [False, True])
+def test_batch_of_tile_passes(fftu, dt, inplace):
+    """One launch over transforms of one to three whole-axis passes, tiny to several thousand points an axis; in
+    complex128 one of them holds values that take FP64 arithmetic."""
+    import torch
+    shapes = [(32, 64, 128), (16,), (2, 2), (4096,), (8, 1024), (128, 32, 32), (64, 4, 4, 16), (1, 256, 2)]
+    xs = [complex_uniform(700 + i, s, dtype=dt) for i, s in enumerate(shapes)]
+    scale = [1.0] * len(xs)
+    if dt == np.complex128:
+        xs[5], scale[5] = xs[5] * 2.0 ** 985, 2.0 ** -900
+    ts = [torch.from_numpy(x).cuda() for x in xs]
+    outs = ts if inplace else [torch.empty_like(t) for t in ts]
+    plans = [fftu.Plan(s, None, dtype=t.dtype) for s, t in zip(shapes, ts)]
+    b = fftu.fftu_batch_create([p.handle for p in plans])
+    fftu.fftu_batch_exec(b, [t.data_ptr() for t in ts], [o.data_ptr() for o in outs],
+                         torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    fftu.fftu_batch_check_status(b)
+    fftu.fftu_batch_destroy(b)
+    for p in plans:
+        p.close()
+    for x, o, s in zip(xs, outs, scale):
+        assert oracle.rel_l2(o.cpu().numpy() * s, oracle.fftn(x.astype(np.complex128) * s)) <= tol(dt, x.size)
