@@ -140,6 +140,7 @@ struct TileStage {
     int lo, lg_q;       // twiddle column q in [2^lg_q]: kind 1 j = tile bits [lo, lo + lg_q); kind 2 class s = tile bits
                         // [lo, lo + lg_p) and the axis' bits above the digit
     int lg_p, lg_step;  // kind 1: exponent r j 2^lg_step; kind 2: exponent (k_prev + r 2^lg_step) s
+    int sh;             // complex128: log2 of the next stage's points (its values are scaled down by them)
     int nk;             // kind 2: k_prev = fields k[] of the bits above the digit
     BitField k[2];
     int tab;            // the table's place in shared memory (elements): entry (r, q) at tab + (r << lg_q) + q

@@ -7,12 +7,16 @@
 // sub-DFT mixes is brought to a common exponent E (that of its largest component), held as signed 64-bit
 // integers through all its stages, and rounded back to FP64 once at the end.
 //
-// Scale: a component x becomes x 2^(K - (E - 1023)), |x| < 2^(E - 1022), with K = 60 - rho for a first stage of
-// 2^rho points, so that after that stage every modulus is below 2^61.5 (2^(K + 1.5) grown by 2^rho); each later
-// stage of 2^rho points first shifts right by rho (rounding), which restores the same bound.  Roundings are
-// half a unit at 2^(K) = 2^57 or more of the largest input, against 2^53 for FP64: the error is below FP64's.
-// Twiddles are Q62 (+1 is 1 - 2^-62); a product keeps the high 64 bits, the low x low partial product
+// Scale: a component x becomes x 2^(K - (E - 1023)), |x| < 2^(E - 1022), with K = 59 - rho for a first stage of
+// 2^rho points, so that after that stage every modulus is below 2^60.5 (2^(K + 1.5) grown by 2^rho); before each
+// later stage of 2^rho points the values are scaled down by 2^rho (rounding), which restores the same bound.
+// Roundings are about a unit at 2^K = 2^56 or more of the largest input, against 2^53 for FP64: the error is below
+// FP64's.  Twiddles are Q62 (+1 is 1 - 2^-62); a product keeps the high 64 bits, the low x low partial product
 // being left out (its mean is added as a constant).
+//
+// The way back to FP64 is the conversion instruction (2 per clock and SM, on the otherwise idle FP64 unit) and an
+// integer addition to the exponent; done in integer instructions it took 44 of a complex value's 271 in a two-stage
+// pass and the integer pipe was the bound.
 //
 // A group with a component that is infinite, NaN, or too small or large to be scaled (fx_plain) is left to the
 // FP64 path of the caller.
@@ -51,6 +55,8 @@ __device__ __forceinline__ int fx_exp(int key) {
     return e > kFxMinExp ? e : kFxMinExp;
 }
 
+constexpr int kFxTop = 59;  // K + rho of the first stage
+
 // x 2^(K - (E - 1023)), truncated toward zero (unbiased for data of both signs); |x| < 2^(E - 1022).
 // K in [52, 62).
 template <int K> __device__ __forceinline__ long long fx_in(double x, int E) {
@@ -68,25 +74,14 @@ template <int K> __device__ __forceinline__ long long fx_in(double x, int E) {
     return (m ^ s) - s;
 }
 
-// The double nearest to v 2^(e0 - 1023 - 63) (round half up in magnitude); v = 0 gives +0.
-__device__ __forceinline__ double fx_out(long long v, int e0) {
-    const int s = (int)(v >> 63);
-    const unsigned long long m = (unsigned long long)((v ^ (long long)s) - (long long)s);
-    unsigned h = (unsigned)(m >> 32), l = (unsigned)m;
-    const bool small = h == 0;
-    h = small ? l : h;
-    l = small ? 0u : l;
-    const int z = __clz((int)h);
-    const unsigned nh = __funnelshift_l(l, h, z), nl = l << (z & 31);
-    unsigned long long r = ((unsigned long long)nh << 32) | nl;
-    // 53 bits and the rounding bit; the implicit one adds 1 to the exponent field
-    const unsigned rb = (nl >> 10) & 1u;
-    const int e = e0 - z - (small ? 32 : 0) - 1;
-    r = (r >> 11) + rb;
-    const unsigned oh = (unsigned)(r >> 32) + ((unsigned)e << 20);
-    double out = __hiloint2double((int)(oh | ((unsigned)s & 0x80000000u)), (int)(unsigned)r);
-    return m == 0 ? 0.0 : out;
+// The double nearest to v 2^e (normal results); v = 0 gives +0.
+__device__ __forceinline__ double fx_out(long long v, int e) {
+    const double y = __ll2double_rn(v);
+    const int hi = __double2hiint(y);
+    return __hiloint2double(hi == 0 ? 0 : hi + (e << 20), __double2loint(y));
 }
+// Exponent of the results of a DFT of 2^lg points whose inputs were scaled with E.
+__device__ __forceinline__ int fx_out_exp(int E, int lg) { return E - 1023 - kFxTop + lg; }
 
 // Twiddle in Q62, each part as hi 2^31 + lo with 0 <= lo < 2^31: (re hi, re lo, im hi, im lo).
 __device__ __forceinline__ int2 fx_q62(double w) {
@@ -95,26 +90,32 @@ __device__ __forceinline__ int2 fx_q62(double w) {
     return make_int2((int)(q >> 31), (int)(q & 0x7fffffff));
 }
 
-// a w (forward) or a conj(w) (inverse); |a| < 2^61.5.
+// a w (forward) or a conj(w) (inverse); |a| < 2^60.5, so that both cross products fit one accumulator.
 template <int DIR> __device__ __forceinline__ longlong2 fx_cmul(longlong2 a, int4 w) {
     const int rh = (int)(a.x >> 31), rl = (int)(a.x & 0x7fffffff);
     const int ih = (int)(a.y >> 31), il = (int)(a.y & 0x7fffffff);
     constexpr long long half = 1ll << 30;
-    long long A, M, N;
     longlong2 r;
     // re = ar wr - ai wi (forward), ar wr + ai wi (inverse)
     const int sih = DIR < 0 ? -ih : ih, sil = DIR < 0 ? -il : il;
-    A = (long long)rh * w.x + (long long)sih * w.z;
-    M = (long long)rh * w.y + (long long)sih * w.w + half;
-    N = (long long)rl * w.x + (long long)sil * w.z + half + (DIR < 0 ? 0 : half);
-    r.x = A + (M >> 31) + (N >> 31);
+    long long A = (long long)rh * w.x + (long long)sih * w.z;
+    long long M = (long long)rh * w.y + (long long)sih * w.w + (long long)rl * w.x + (long long)sil * w.z + half +
+                  (DIR < 0 ? 0 : half);
+    r.x = A + (M >> 31);
     // im = ai wr + ar wi (forward), ai wr - ar wi (inverse)
     const int srh = DIR < 0 ? rh : -rh, srl = DIR < 0 ? rl : -rl;
     A = (long long)ih * w.x + (long long)srh * w.z;
-    M = (long long)ih * w.y + (long long)srh * w.w + half;
-    N = (long long)il * w.x + (long long)srl * w.z + half + (DIR < 0 ? half : 0);
-    r.y = A + (M >> 31) + (N >> 31);
+    M = (long long)ih * w.y + (long long)srh * w.w + (long long)il * w.x + (long long)srl * w.z + half +
+        (DIR < 0 ? half : 0);
+    r.y = A + (M >> 31);
     return r;
+}
+// The twiddle w 2^-sh.
+__device__ __forceinline__ int4 fx_scale_tw(int4 w, int sh) {
+    if (sh == 0) return w;
+    const long long half = 1ll << (sh - 1);
+    const long long re = (((long long)w.x << 31) + w.y + half) >> sh, im = (((long long)w.z << 31) + w.w + half) >> sh;
+    return make_int4((int)(re >> 31), (int)(re & 0x7fffffff), (int)(im >> 31), (int)(im & 0x7fffffff));
 }
 // a c for a constant c > 0 in Q62.
 template <long long C> __device__ __forceinline__ long long fx_mulc(long long a) {
@@ -199,10 +200,10 @@ template <int R, int DIR> __device__ __forceinline__ void fx_dft(longlong2 *v) {
     }
 }
 
-// Shift of a later stage of 2^RHO points (rounding).
-template <int RHO> __device__ __forceinline__ longlong2 fx_scale_down(longlong2 a) {
-    constexpr long long half = RHO > 0 ? 1ll << (RHO > 0 ? RHO - 1 : 0) : 0;
-    return mk<longlong2>((a.x + half) >> RHO, (a.y + half) >> RHO);
+// a 2^-sh (rounding).
+__device__ __forceinline__ longlong2 fx_scale_down(longlong2 a, int sh) {
+    const long long half = (1ll << sh) >> 1;
+    return mk<longlong2>((a.x + half) >> sh, (a.y + half) >> sh);
 }
 
 template <int R> __host__ __device__ constexpr int lg_of() { return R == 2 ? 1 : R == 4 ? 2 : R == 8 ? 3 : R == 16 ? 4 : R == 32 ? 5 : 0; }

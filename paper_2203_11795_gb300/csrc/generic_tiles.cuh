@@ -332,7 +332,7 @@ __device__ __forceinline__ bool fx_stage(longlong2 *sm, const int4 *__restrict__
                 const int k = b & (Ns - 1);
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
-                    longlong2 x = fx_scale_down<RHO>(sm[smi(base + (b + r * per_col) * js, a.swz)]);
+                    longlong2 x = fx_scale_down(sm[smi(base + (b + r * per_col) * js, a.swz)], RHO);
                     if (r > 0) x = fx_cmul<DIR>(x, tw[r * k * twstep]);
                     v[q][r] = x;
                 }
@@ -357,7 +357,7 @@ __device__ __forceinline__ bool fx_stage(longlong2 *sm, const int4 *__restrict__
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     const double2 x = fx_bits(v[q][r]);
-                    v[q][r] = mk<longlong2>(fx_in<60 - RHO>(x.x, E), fx_in<60 - RHO>(x.y, E));
+                    v[q][r] = mk<longlong2>(fx_in<kFxTop - RHO>(x.x, E), fx_in<kFxTop - RHO>(x.y, E));
                 }
                 fx_dft<R, DIR>(v[q]);
             }
@@ -395,9 +395,8 @@ __device__ __forceinline__ void axis_tile_fx(const AxisPass &a, int64_t t, doubl
         return;
     }
     for (; Ns < a.len; Ns *= 8) fx_stage<DIR, 8, false>(fx, tw, a, Ns, emax, tid, nt);
-    // after the first stage 2^K = 2^60 / R0, each later stage one factor lower: 2^60 / len in all; 1/N is a
-    // power of two and goes into the exponent
-    const int e_add = 3 + a.lg_len + (__double2hiint(a.scale) >> 20) - 1023;
+    // 1/N is a power of two and goes into the exponent
+    const int lg_scale = (__double2hiint(a.scale) >> 20) - 1023;
     for (int e = tid; e < a.tile; e += nt) {
         int lpo, v;
         if (a.contiguous) {
@@ -425,7 +424,7 @@ __device__ __forceinline__ void axis_tile_fx(const AxisPass &a, int64_t t, doubl
         }
         const int key = emax[a.contiguous ? (v << a.lg_Gt) + cl : (cl << a.lg_V) + v];
         if (key == 0) x = mk<longlong2>(0, 0);  // all zeros: no trace of the products' rounding constants
-        const int e0 = fx_exp(key) + e_add;
+        const int e0 = fx_out_exp(fx_exp(key), a.lg_len) + lg_scale;
         const int64_t g = a.contiguous ? o.gbase + (int64_t)v * a.nl + gp : o.gbase + gp * a.inner + v;
         dst[g] = mk<double2>(fx_out(x.x, e0), fx_out(x.y, e0));
     }
@@ -474,7 +473,7 @@ template <int DIR, int LO, int HI> __device__ __forceinline__ void fiber_dft(dou
     const int E = fx_exp(key);
     longlong2 x[PG];
 #pragma unroll
-    for (int j = 0; j < PG; ++j) x[j] = mk<longlong2>(fx_in<60 - RHO>(v[j].x, E), fx_in<60 - RHO>(v[j].y, E));
+    for (int j = 0; j < PG; ++j) x[j] = mk<longlong2>(fx_in<kFxTop - RHO>(v[j].x, E), fx_in<kFxTop - RHO>(v[j].y, E));
 #pragma unroll
     for (int jh = 0; jh < HI; ++jh) fx_dft<LO, DIR>(x + jh * LO);
     if constexpr (HI > 1) {
@@ -488,7 +487,7 @@ template <int DIR, int LO, int HI> __device__ __forceinline__ void fiber_dft(dou
             for (int jh = 0; jh < HI; ++jh) x[jh * LO + jl] = w[jh];
         }
     }
-    const int e0 = E + 3 + RHO + lg_scale;
+    const int e0 = fx_out_exp(E, RHO) + lg_scale;
 #pragma unroll
     for (int j = 0; j < PG; ++j) v[j] = mk<double2>(fx_out(x[j].x, e0), fx_out(x[j].y, e0));
 }

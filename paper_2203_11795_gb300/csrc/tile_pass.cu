@@ -270,6 +270,7 @@ bool make_tile_pass(int d, const int64_t *n, const int64_t *p, int l0, int l1, i
         TileStage &s = a.st[si];
         s.lg_r = g.bits;
         s.pos = g.pos;
+        s.sh = si + 1 < no ? dg[order[si + 1]].bits : 0;
         s.tw = tw[l];
         s.tw64 = tw64[l];
         for (int r = 0; r < 1 << g.bits; ++r) s.rx[r] = slot(r << g.pos);

@@ -166,17 +166,14 @@ __device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_
                 const int E = fx_exp(key);
 #pragma unroll
                 for (int r = 0; r < R; ++r)
-                    v[r] = mk<longlong2>(fx_in<60 - RHO>(x[r].x, E), fx_in<60 - RHO>(x[r].y, E));
+                    v[r] = mk<longlong2>(fx_in<kFxTop - RHO>(x[r].x, E), fx_in<kFxTop - RHO>(x[r].y, E));
             } else {
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[r] = tp_load<OPT>(p + ((size_t)r << a.in_bit));
             }
         } else {
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                v[r] = sm[slot ^ s.rx[r]];
-                if constexpr (ARITH == kTpFixed) v[r] = fx_scale_down<RHO>(v[r]);
-            }
+            for (int r = 0; r < R; ++r) v[r] = sm[slot ^ s.rx[r]];
         }
         tp_dft<ARITH, DIR, R>(v);
         if constexpr (LAST) {
@@ -190,7 +187,7 @@ __device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_
                 q = dst + tp_fields(a.out, a.nout, (unsigned)phi);
             }
             if constexpr (ARITH == kTpFixed && !FIRST) key = emax[tp_fields(a.group, a.ngroup, (unsigned)e0)];
-            [[maybe_unused]] const int x0 = fx_exp(key) + 3 + a.lg_dft + a.lg_scale;
+            [[maybe_unused]] const int x0 = fx_out_exp(fx_exp(key), a.lg_dft) + a.lg_scale;
             [[maybe_unused]] const auto f = (typename real_of<W>::type)a.scale;
             // kTpMul: the pointwise factor at the same natural index
             [[maybe_unused]] const typename T::elem *m =
@@ -209,6 +206,14 @@ __device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_
             }
         } else {
             if (s.tw_kind) tp_twiddles<ARITH, DIR, OPT, R>(s, e0, v, tabs);
+            if constexpr (ARITH == kTpFixed) {  // the next stage's scale, where the table did not bring it
+                if ((OPT & kTpGlobalTw) != 0 || s.tw_kind == 0) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) v[r] = fx_scale_down(v[r], s.sh);
+                } else if (s.tw_kind == 1) {
+                    v[0] = fx_scale_down(v[0], s.sh);
+                }
+            }
 #pragma unroll
             for (int r = 0; r < R; ++r) sm[slot ^ s.rx[r]] = v[r];
         }
@@ -247,8 +252,11 @@ __device__ __forceinline__ void tp_tables(const TilePass &a, typename tp_type<AR
         if (s.tw_kind == 0) continue;
         const TW *tw = static_cast<const TW *>(s.tw);
         const int n = 1 << (s.lg_r + s.lg_q);
-        for (int i = threadIdx.x; i < n; i += blockDim.x)
-            tabs[s.tab + i] = tw[tp_exponent(s, (unsigned)i >> s.lg_q, (unsigned)i & ((1u << s.lg_q) - 1))];
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            const TW w = tw[tp_exponent(s, (unsigned)i >> s.lg_q, (unsigned)i & ((1u << s.lg_q) - 1))];
+            if constexpr (ARITH == kTpFixed) tabs[s.tab + i] = fx_scale_tw(w, s.sh);
+            else tabs[s.tab + i] = w;
+        }
     }
 }
 
