@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(const __grid_const
 // the strided kernel's 3 or 4, each with fewer trips through shared memory).
 struct TileJob {
     int transform, dep;
-    int64_t first, dep_tiles;
+    int64_t dep_tiles;
     TilePass a;
 };
 
@@ -165,68 +165,95 @@ struct TileParams {
 
 constexpr int kTileBatchThreads = 256;
 
-// The tasks in order with their bounded waits as in batch_kernel.  Twiddles come straight from the root tables (a CTA's
-// next tile is usually another job's).  Four CTAs per SM for complex64 (64 registers), three for complex128 (80).
+// The tasks in order with their bounded waits as in batch_kernel.  A CTA holds its current and its next task: while the
+// current tile computes, the next one's job descriptor comes in and the one after is claimed, so that neither the atomic
+// nor the lookups are waited for.  The earliest unfinished task is always some CTA's current one (a next task is later
+// than its CTA's current one), so it can run.  Twiddles come straight from the root tables (a CTA's next tile is usually
+// another job's).  Four CTAs per SM (64 registers).
 template <int ARITH, int DIR>
-__global__ void __launch_bounds__(kTileBatchThreads, ARITH == kTpF32 ? 4 : 3)
+__global__ void __launch_bounds__(kTileBatchThreads, 4)
     tile_batch_kernel(const __grid_constant__ TileParams P, int emax_off) {
     using T = tp_type<ARITH>;
     using E = typename T::elem;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     auto *sm = reinterpret_cast<typename T::work *>(smem_raw);
     int *emax = reinterpret_cast<int *>(smem_raw + emax_off);
-    __shared__ __align__(16) TileJob s_job;
-    __shared__ long long s_task;
-    __shared__ int s_jobi, s_ok, s_loaded;
+    __shared__ __align__(16) TileJob s_job[2];
+    __shared__ int s_firsts[kMaxBatchJobs];  // task indices fit 31 bits
+    __shared__ int s_task[2], s_jobi[2], s_ok;
     const int tid = threadIdx.x;
-    if (tid == 0) s_loaded = -1;
+    for (int j = tid; j < P.njobs; j += blockDim.x) s_firsts[j] = (int)P.firsts[j];
+    if (tid == 0) s_task[0] = (int)atomicAdd(P.task_ctr, 1ull);
     __syncthreads();
-    for (;;) {
-        if (tid == 0) {
-            const long long t = (long long)atomicAdd(P.task_ctr, 1ull);
-            s_task = t;
-            if (t < P.total) {
-                int lo = 0, hi = P.njobs - 1;  // last job with first <= t
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (__ldg(P.firsts + mid) <= t) lo = mid;
-                    else hi = mid - 1;
-                }
-                s_jobi = lo;
-            }
+    auto find_job = [&](int t) {
+        int lo = 0, hi = P.njobs - 1;  // last job with first <= t
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (s_firsts[mid] <= t) lo = mid;
+            else hi = mid - 1;
         }
-        __syncthreads();
-        const long long t = s_task;
+        return lo;
+    };
+    constexpr int kWords = (int)(sizeof(TileJob) / sizeof(int));
+    auto load_job = [&](int slot, int j) {
+        const int *srcw = reinterpret_cast<const int *>(P.jobs + j);
+        int *dstw = reinterpret_cast<int *>(&s_job[slot]);
+        for (int w = tid; w < kWords; w += blockDim.x) {
+            const unsigned d = (unsigned)__cvta_generic_to_shared(dstw + w);
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(srcw + w) : "memory");
+        }
+    };
+    if (s_task[0] < P.total) {
+        const int j = find_job(s_task[0]);
+        if (tid == 0) s_jobi[0] = j;
+        load_job(0, j);
+    }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    if (tid == 0) s_task[1] = (int)atomicAdd(P.task_ctr, 1ull);
+    __syncthreads();
+    for (int slot = 0;; slot ^= 1) {
+        const int t = s_task[slot];
         if (t >= P.total) break;
-        const int j = s_jobi;
-        if (j != s_loaded) {
-            const int *srcw = reinterpret_cast<const int *>(P.jobs + j);
-            int *dstw = reinterpret_cast<int *>(&s_job);
-            for (int w = tid; w < (int)(sizeof(TileJob) / sizeof(int)); w += blockDim.x) dstw[w] = srcw[w];
+        const TilePass &a = s_job[slot].a;
+        const int j = s_jobi[slot];
+        // the next task's descriptor, under way during this tile
+        const int tn = s_task[slot ^ 1];
+        if (tn < P.total) {
+            const int jn = find_job(tn);
+            if (tid == 0) s_jobi[slot ^ 1] = jn;
+            load_job(slot ^ 1, jn);
         }
-        __syncthreads();
-        const TilePass &a = s_job.a;
         if (tid == 0) {
-            s_loaded = j;
-            const int dep = s_job.dep;
-            s_ok = dep < 0 || wait_counter_geq(P.done + dep, (unsigned)s_job.dep_tiles, P.spin_limit_ns, P.status);
+            const int dep = s_job[slot].dep;
+            s_ok = dep < 0 || wait_counter_geq(P.done + dep, (unsigned)s_job[slot].dep_tiles, P.spin_limit_ns, P.status);
         }
         if constexpr (ARITH == kTpFixed)
             for (int i = tid; i < 1 << a.lg_groups; i += blockDim.x) emax[i] = 0;
         __syncthreads();
+        int claimed = 0;
+        if (tid == 0 && tn < P.total) claimed = (int)atomicAdd(P.task_ctr, 1ull);  // used after the tile
         if (s_ok) {
-            const int64_t base = tp_base(a, t - s_job.first);
-            E *out = static_cast<E *>(P.out[s_job.transform]) + base;
-            const E *src = s_job.dep < 0 ? static_cast<const E *>(P.in[s_job.transform]) + base : out;
-            if (!tp_run<ARITH, DIR, kTpGlobalTw>(a, sm, nullptr, emax, src, out)) {
-                if constexpr (ARITH == kTpFixed) tp_run_fp64<DIR, kTpGlobalTw>(a, reinterpret_cast<double2 *>(sm), src, out);
+            const int64_t base = tp_base(a, t - s_firsts[j]);
+            E *out = static_cast<E *>(P.out[s_job[slot].transform]) + base;
+            const E *src = s_job[slot].dep < 0 ? static_cast<const E *>(P.in[s_job[slot].transform]) + base : out;
+            constexpr int kOpt = kTpGlobalTw, kOne = kTpGlobalTw | kTpSingle;
+            const bool done = a.nst == 1 ? tp_run<ARITH, DIR, kOne>(a, sm, nullptr, emax, src, out)
+                                         : tp_run<ARITH, DIR, kOpt>(a, sm, nullptr, emax, src, out);
+            if (ARITH == kTpFixed && !done) {
+                double2 *smd = reinterpret_cast<double2 *>(smem_raw), *o = reinterpret_cast<double2 *>(out);
+                const double2 *i = reinterpret_cast<const double2 *>(src);
+                if (a.nst == 1) tp_run_fp64<DIR, kOne>(a, smd, i, o);
+                else tp_run_fp64<DIR, kOpt>(a, smd, i, o);
             }
         }
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
         __syncthreads();
         if (tid == 0) {
             __threadfence();
             atomicAdd(P.done + j, 1u);
+            s_task[slot] = tn < P.total ? claimed : (int)P.total;  // the task after the next
         }
+        __syncthreads();
     }
 }
 
@@ -395,9 +422,13 @@ fftu_status batch_create(int count, const fftu_handle *plans, Batch **out_batch)
     int64_t first = 0;
     std::vector<int64_t> firsts(njobs);
     for (size_t j = 0; j < njobs; ++j) {
-        (tiles ? tjobs[j].first : jobs[j].first) = first;
+        if (!tiles) jobs[j].first = first;
         firsts[j] = first;
         first += tiles ? tjobs[j].a.tiles : jobs[j].tiles;
+    }
+    if (tiles && first > 0x7fffffffll - 4096) {  // (the kernel's task indices; far beyond device memory)
+        record_error("batch: too many tiles in total");
+        return FFTU_ERR_UNSUPPORTED;
     }
     Batch *b = new (std::nothrow) Batch();
     if (!b) {

@@ -436,19 +436,24 @@ bool make_triple_pass(const Plan &pl, TriplePass &a) {
 // 2048 complex128 elements, up to 64 KB.  Runs on a strided group: complex64 16 elements (128 bytes), 8 where 16 do
 // not fit the tile; complex128 4.  Measured on 512 x 512 x 256 complex64 (floor 158 us a pass): the 512-point axes 214 and
 // 358 us at 8, 192 and 190 us at 16; a 1024-point axis 223-279 us at 8, 246-262 us at 16 with a 128 KB tile.
+// Longer strided axes: 2048 points in 16384-element tiles with runs of 8, 4096 with runs of 4 (64 x 2048 x 512: 287 us
+// for that axis, 627 in all against 849 through line passes and phase B; 32 x 4096 x 512: 329, 664 against 947);
+// contiguous lines up to 4096 points (32 KB of twiddles beside the tile).
 // batched: for a launch that many transforms share (usual tiles whatever N, no radix-32 stages, at most 256 threads).
 bool choose_tile_pass(int d, const int64_t *n, const int64_t *p, int l1, int l_min, int is_double,
                       const void *const *tw, const void *const *tw64, bool batched, int *l0_out, TilePass &a) {
-    const int target = is_double ? 11 : 12, max_tile = is_double ? 12 : 13, min_v = is_double ? 2 : 3;
+    const int target = is_double ? 11 : 12, min_v = is_double ? 2 : 3;
     int64_t inner = 1, N = 1;
     for (int l = 0; l < d; ++l) N *= n[l];
     for (int l = l1 + 1; l < d; ++l) inner *= n[l];
     const bool contiguous = inner == 1;
     const int lg_in = ilog2(inner);
-    const int need_v = contiguous ? 0 : std::min(min_v, lg_in);
-    const int max_g = contiguous ? target : max_tile - need_v;  // several axes
     int l0 = l1, lg_g = ilog2(n[l1]);
-    if (lg_g + need_v > max_tile) return false;
+    // a single long strided axis: tiles of 128 KB (one CTA per SM) and, for 4096 points, runs of 4
+    const int max_tile = (is_double ? 12 : 13) + (!contiguous && lg_g > 10 && !batched ? 1 : 0);
+    const int need_v = contiguous ? 0 : std::min(!is_double && lg_g == 12 ? 2 : min_v, lg_in);
+    const int max_g = contiguous ? target : max_tile - need_v;  // several axes
+    if (lg_g + need_v > max_tile || (contiguous && lg_g > 12)) return false;
     while (l0 > l_min && l1 - l0 < 2 && lg_g + ilog2(n[l0 - 1]) <= max_g) lg_g += ilog2(n[--l0]);
     for (;; ++l0) {  // fewer axes when the stages do not work out
         while (l0 < l1 && n[l0] == 1) ++l0;
@@ -457,7 +462,7 @@ bool choose_tile_pass(int d, const int64_t *n, const int64_t *p, int l1, int l_m
         for (int l = 0; l < l0; ++l) outer *= n[l];
         for (int l = l0; l <= l1; ++l) lg_g += ilog2(n[l]);
         int lg_v = std::max(target - lg_g, need_v);
-        if (!contiguous && !is_double && lg_v == 3 && lg_g + 4 <= max_tile) lg_v = 4;
+        if (!contiguous && !is_double && lg_v == 3 && lg_g + 4 <= 13) lg_v = 4;
         lg_v = std::min(lg_v, contiguous ? ilog2(outer) : lg_in);
         // small arrays: smaller tiles while the GPU is not full
         while (!batched && lg_v > (contiguous ? 0 : need_v) && lg_v + lg_g > 9 && (N >> (lg_g + lg_v)) < 304) --lg_v;

@@ -155,6 +155,7 @@ struct TilePass {
     int64_t tiles;
     int grid, threads;  // persistent grid
     int wide;           // complex64: radix-32 stages
+    int once;           // one stage, one fiber per thread, a barrier between the loads and the stores
     int lg_g, lg_v, lg_inner, lg_tile;  // lg_g: positions of the axes; lg_inner < 0: contiguous
     int lg_dft;                         // log2 of the points of one sub-DFT
     int in_bit, out_bit;                // element-offset bit of the first stage's and the last stage's digit

@@ -11,10 +11,10 @@
 namespace fftu {
 namespace {
 
-// Persistent: the twiddle tables are built once per CTA.  Registers: 64 for complex64 (two CTAs of 512 threads, four of
-// 256), 80 for complex128 (the bound of 768 threads; three CTAs of 256).
+// Persistent: the twiddle tables are built once per CTA.  64 registers (1024 threads per SM, in CTAs of 256 for the usual
+// tiles), 128 with radix-32 stages.
 template <int ARITH, int DIR, int OPT>
-__global__ void __launch_bounds__(ARITH == kTpF32 ? 512 : ARITH == kTpF32w ? 256 : 768, ARITH == kTpFixed ? 1 : 2) tile_pass_kernel(const __grid_constant__ TilePass a) {
+__global__ void __launch_bounds__(ARITH == kTpF32w ? 512 : 1024) tile_pass_kernel(const __grid_constant__ TilePass a) {
     using T = tp_type<ARITH>;
     using E = typename T::elem;
     extern __shared__ __align__(128) unsigned char tp_raw[];
@@ -94,22 +94,31 @@ cudaError_t launch_t(const TilePass &a, cudaStream_t st) {
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return a.mul ? cudaLaunchKernelEx(&cfg, tile_pass_kernel<ARITH, DIR, kTpMul>, a)
-                 : cudaLaunchKernelEx(&cfg, tile_pass_kernel<ARITH, DIR, 0>, a);
+    switch ((a.mul ? kTpMul : 0) | (a.nst == 1 ? kTpSingle : 0)) {
+        case 0: return cudaLaunchKernelEx(&cfg, tile_pass_kernel<ARITH, DIR, 0>, a);
+        case kTpMul: return cudaLaunchKernelEx(&cfg, tile_pass_kernel<ARITH, DIR, kTpMul>, a);
+        case kTpSingle: return cudaLaunchKernelEx(&cfg, tile_pass_kernel<ARITH, DIR, kTpSingle>, a);
+        default: return cudaLaunchKernelEx(&cfg, tile_pass_kernel<ARITH, DIR, kTpMul | kTpSingle>, a);
+    }
+}
+
+template <int ARITH, int DIR, int OPT>
+cudaError_t prepare_opt(const TilePass &a, int *per_sm) {
+    cudaError_t e = cudaFuncSetAttribute(tile_pass_kernel<ARITH, DIR, OPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kMaxDynSmem);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, tile_pass_kernel<ARITH, DIR, OPT>, a.threads, a.smem);
 }
 
 template <int ARITH, int DIR>
 cudaError_t prepare_t(TilePass &a) {
-    cudaError_t e = cudaFuncSetAttribute(tile_pass_kernel<ARITH, DIR, 0>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+    int dev = 0, sms = 0, per_sm = 0, other = 0;
+    cudaError_t e = a.nst == 1 ? prepare_opt<ARITH, DIR, kTpMul | kTpSingle>(a, &other)
+                               : prepare_opt<ARITH, DIR, kTpMul>(a, &other);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tile_pass_kernel<ARITH, DIR, kTpMul>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kMaxDynSmem);
-    int dev = 0, sms = 0, per_sm = 0;
+        e = a.nst == 1 ? prepare_opt<ARITH, DIR, kTpSingle>(a, &per_sm) : prepare_opt<ARITH, DIR, 0>(a, &per_sm);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tile_pass_kernel<ARITH, DIR, 0>, a.threads, a.smem);
     if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
     a.grid = sms * per_sm;
     return e;
@@ -153,7 +162,9 @@ bool make_tile_pass(int d, const int64_t *n, const int64_t *p, int l0, int l1, i
             dig[0] = bits - dig[1];
             k = 2;
         }
-        if (p && l0 == l1 && k == 1 && lg_p[l] > 0) {  // the Put moves s: loads and stores need a barrier between them
+        // one digit in phase A: the Put moves s, so loads and stores need a barrier between them.  A strided axis takes
+        // one fiber per thread and a barrier in its only stage; contiguous lines two stages (lanes along memory).
+        if (p && l0 == l1 && k == 1 && lg_p[l] > 0 && contiguous) {
             if (bits < 2) return false;
             dig[1] = bits / 2;
             dig[0] = bits - dig[1];
@@ -177,6 +188,7 @@ bool make_tile_pass(int d, const int64_t *n, const int64_t *p, int l0, int l1, i
     for (int i = 1; i < count_of[l0]; ++i) order[no++] = first_of[l0] + i;
     if (no == 0) return false;
     if (no == 1 && p && l1 > l0) return false;  // (axes of length 2 beside it: left to the strided pass)
+    a.once = no == 1 && p && lg_p[l0] > 0;
     a.nst = no;
     // output position of every tile bit (element-offset bits, relative to the tile's base): an axis' first (highest)
     // digit holds the lowest bits of k; the class s goes above k
@@ -202,7 +214,7 @@ bool make_tile_pass(int d, const int64_t *n, const int64_t *p, int l0, int l1, i
     int tb[32], nt = 0;
     for (int b = 0; b < a.lg_tile; ++b)
         if (b < dl.pos || b >= dl.pos + dl.bits) tb[nt++] = b;
-    for (int i = 1; i < nt; ++i)
+    for (int i = 1; i < nt && no > 1; ++i)  // (a single stage keeps the order of its loads)
         for (int k = i; k > 0 && out_bit[tb[k - 1]] > out_bit[tb[k]]; --k) std::swap(tb[k - 1], tb[k]);
     for (int i = 0; i < nt;) {
         int j = i + 1;
@@ -301,7 +313,8 @@ bool make_tile_pass(int d, const int64_t *n, const int64_t *p, int l0, int l1, i
     a.smem = a.emax_off + (is_double ? sizeof(int) << a.lg_groups : 0);
     // complex128: one fiber of the first stage per thread (its exponent covers all of them); complex64: 16 values
     a.threads = is_double ? 1 << (a.lg_tile - a.st[0].lg_r) : a.lg_tile > 9 + wide ? 1 << (a.lg_tile - 4 - wide) : 32;
-    if (a.threads > (wide ? 256 : 512) || a.smem > (size_t)kMaxDynSmem) return false;
+    if (a.once) a.threads = 1 << (a.lg_tile - a.st[0].lg_r);
+    if (a.threads > (wide ? 512 : 1024) || a.smem > (size_t)kMaxDynSmem) return false;
     a.scale = 1.0;
     return true;
 }

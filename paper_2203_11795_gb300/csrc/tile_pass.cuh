@@ -11,6 +11,7 @@
 // V = 2^lg_v adjacent inner positions (inner > 1) or V adjacent outer positions (inner = 1, contiguous memory).
 // Tile index e: [g][v] or [v][g], g row-major over the axes, so tile order is memory order.  Each axis is split
 // into digits of at most 5 bits, highest first; a stage transforms one digit in place:
+// A pass of one stage stores from the registers it loaded into (phase A: after a barrier).
 //   x[j + T r] (j in [T]: the axis' lower digits) -> F_R over r -> k in the digit's place, times w_{R T}^{k j}.
 // In phase A the digits split m (i = s + p m) and s, the lowest bits of the axis, stays in place until the store.
 // The first stage loads its fibers from HBM into registers and the last one stores them to HBM, with the digits
@@ -36,8 +37,8 @@ namespace fftu {
 // ARITH of a tile pass; kTpF32w: complex64 with radix-32 stages (a kernel of its own, with twice the registers)
 constexpr int kTpF32 = 0, kTpFixed = 1, kTpF64 = 2, kTpF32w = 3;
 // OPT bits: the pointwise product in the last store; twiddles straight from the root tables (many kinds of pass in one
-// launch) instead of the stages' shared tables
-constexpr int kTpMul = 1, kTpGlobalTw = 2;
+// launch) instead of the stages' shared tables; a pass of one stage.
+constexpr int kTpMul = 1, kTpGlobalTw = 2, kTpSingle = 4;
 template <int ARITH> struct tp_type;
 template <> struct tp_type<kTpF32> { using elem = float2; using work = float2; using tw = float2; };
 template <> struct tp_type<kTpF32w> : tp_type<kTpF32> {};
@@ -180,12 +181,9 @@ __device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_
             if (s.tw_kind) tp_twiddles<ARITH, DIR, OPT, R>(s, e0, v, tabs);  // phase A: w_n^{k s} of the last axis
             typename T::elem *q;
             if constexpr (FIRST) {
-                const unsigned off = a.lg_inner < 0 ? (unsigned)e0
-                                                    : (((unsigned)e0 >> a.lg_v) << a.lg_inner) | (e0 & ((1 << a.lg_v) - 1));
-                q = dst + off;
-            } else {
-                q = dst + tp_fields(a.out, a.nout, (unsigned)phi);
+                if (a.once) __syncthreads();  // every thread has one fiber: all loads of the tile are done
             }
+            q = dst + tp_fields(a.out, a.nout, (unsigned)phi);
             if constexpr (ARITH == kTpFixed && !FIRST) key = emax[tp_fields(a.group, a.ngroup, (unsigned)e0)];
             [[maybe_unused]] const int x0 = fx_out_exp(fx_exp(key), a.lg_dft) + a.lg_scale;
             [[maybe_unused]] const auto f = (typename real_of<W>::type)a.scale;
@@ -264,7 +262,7 @@ template <int ARITH, int DIR, int OPT>
 __device__ __forceinline__ bool tp_run(const TilePass &a, typename tp_type<ARITH>::work *sm,
                                        const typename tp_type<ARITH>::tw *tabs, int *emax,
                                        const typename tp_type<ARITH>::elem *src, typename tp_type<ARITH>::elem *dst) {
-    if (a.nst == 1) return tp_stage_any<ARITH, DIR, OPT, true, true>(a, 0, sm, tabs, emax, src, dst);
+    if constexpr ((OPT & kTpSingle) != 0) return tp_stage_any<ARITH, DIR, OPT, true, true>(a, 0, sm, tabs, emax, src, dst);
     if (!tp_stage_any<ARITH, DIR, OPT, true, false>(a, 0, sm, tabs, emax, src, dst)) return false;
     __syncthreads();
     for (int si = 1; si + 1 < a.nst; ++si) {

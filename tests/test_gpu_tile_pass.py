@@ -14,7 +14,7 @@ from fftu_inputs import complex_uniform
 
 pytestmark = pytest.mark.gpu
 
-WHOLE = [(2,), (16,), (32,), (8192,), (4, 2), (2, 2, 2), (16, 16), (8, 4096), (1024, 4), (1024, 1024), (64, 64, 64),
+WHOLE = [(2,), (16,), (32,), (4096,), (4, 2), (2, 2, 2), (16, 16), (8, 4096), (1024, 4), (1024, 1024), (64, 64, 64),
          (32, 2, 128), (128, 32, 256), (1, 64, 1, 512), (16, 8, 4, 4, 2), (32, 32, 32, 32), (512, 2, 16)]
 GRIDS = [((256, 256), (8, 8)), ((1024, 64), (4, 4)), ((64, 128, 32), (4, 8, 2)), ((512, 32, 32), (16, 4, 1)),
          ((8, 1024), (2, 16)), ((4096, 8), (4, 1)), ((16, 16, 128), (2, 4, 8)), ((2048,), (32,)), ((128, 4, 16), (8, 2, 4))]
