@@ -692,10 +692,10 @@ fftu_status build_schedule(Plan &pl, int sched) {
             pl.phase_b.push_back(t);
         }
     }
-    // the library's own choice of grid and schedule: the whole transform by whole-axis passes, except where the ring
-    // phase A applies
-    const bool ring = fused_a && pl.phase_a[0].a3.mode == 1;
-    if (pl.free_grid && sched == FFTU_SCHED_AUTO && pl.precision == FFTU_PREC_NATIVE && !ring) {
+    // the library's own choice of grid and schedule: the whole transform by whole-axis passes, except where the fused phase
+    // A applies (512^3: 2 HBM round trips against 3; 1024^3: 11.7 against 13.1 ms, its strided passes of 1024 points
+    // running at half the copy rate).  On a caller's grid fftu_exec gives what its two phases give, bit for bit.
+    if (pl.free_grid && sched == FFTU_SCHED_AUTO && pl.precision == FFTU_PREC_NATIVE && !fused_a) {
         fftu_status st = build_whole(pl);
         if (st != FFTU_OK) return st;
     }
