@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -147,13 +148,21 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(const __grid_const
 struct TileJob {
     int transform, dep;
     int64_t dep_tiles;
-    TilePass a;
+    TileTask a;
 };
+static_assert(offsetof(TileTask, st) == offsetof(TilePass, st));
+void fill_task(const TilePass &p, TileTask &t) {
+    std::memcpy(static_cast<void *>(&t), &p, offsetof(TilePass, st));
+    for (int i = 0; i < kTpStages; ++i) t.st[i] = p.st[i];
+}
 
 struct TileParams {
     const TileJob *jobs;
     const int64_t *firsts;
+    const int *tab_at;  // job j's twiddle tables (stage after stage, as in a tile pass): 16-byte units [tab_at[j], tab_at[j + 1])
+    const int4 *tabs;
     int njobs;
+    int emax_off, tab_off, tab_units;  // shared memory: exponents, two tables of at most tab_units
     int64_t total;
     unsigned long long *task_ctr;
     unsigned *done;
@@ -164,25 +173,39 @@ struct TileParams {
 };
 
 constexpr int kTileBatchThreads = 256;
+// The jobs' tables are copied to shared memory with their descriptors up to this size (four CTAs of 32 KB tiles per SM);
+// with a longer table in the batch (axes of 512 points and more) its passes read the roots instead.
+constexpr int kTileBatchTable = 512;  // 16-byte units
+
+template <int ARITH>
+__global__ void tile_tables_kernel(const TileJob *jobs, const int *tab_at, int4 *tabs) {
+    tp_tables<ARITH>(jobs[blockIdx.x].a, reinterpret_cast<typename tp_type<ARITH>::tw *>(tabs + tab_at[blockIdx.x]));
+}
 
 // The tasks in order with their bounded waits as in batch_kernel.  A CTA holds its current and its next task: while the
 // current tile computes, the next one's job descriptor comes in and the one after is claimed, so that neither the atomic
 // nor the lookups are waited for.  The earliest unfinished task is always some CTA's current one (a next task is later
-// than its CTA's current one), so it can run.  Twiddles come straight from the root tables (a CTA's next tile is usually
-// another job's).  Four CTAs per SM (64 registers).
-template <int ARITH, int DIR>
-__global__ void __launch_bounds__(kTileBatchThreads, 4)
-    tile_batch_kernel(const __grid_constant__ TileParams P, int emax_off) {
+// than its CTA's current one), so it can run.  A CTA's next tile is usually another job's: TABS: its twiddle tables, made
+// when the batch is created, come in with the descriptor.  Four CTAs per SM (64 registers).  64 uneven complex64 transforms
+// of sides 32 to 128 (28 M elements, 66 us a round trip at the copy rate, two or three passes each): 302 us
+// with twiddles from the roots and 32 slot constants a stage (92 thread instructions per element and pass, a quarter of them
+// shared-memory reads of the descriptor), 244 us with tables and one slot constant per bit (TpSlots).
+template <int ARITH, int DIR, bool TABS>
+__global__ void __launch_bounds__(kTileBatchThreads, 4) tile_batch_kernel(const __grid_constant__ TileParams P) {
     using T = tp_type<ARITH>;
     using E = typename T::elem;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     auto *sm = reinterpret_cast<typename T::work *>(smem_raw);
-    int *emax = reinterpret_cast<int *>(smem_raw + emax_off);
+    int *emax = reinterpret_cast<int *>(smem_raw + P.emax_off);
+    int4 *stabs = reinterpret_cast<int4 *>(smem_raw + P.tab_off);
     __shared__ __align__(16) TileJob s_job[2];
     __shared__ int s_firsts[kMaxBatchJobs];  // task indices fit 31 bits
+    __shared__ int s_tab_at[TABS ? kMaxBatchJobs + 1 : 1];
     __shared__ int s_task[2], s_jobi[2], s_ok;
     const int tid = threadIdx.x;
     for (int j = tid; j < P.njobs; j += blockDim.x) s_firsts[j] = (int)P.firsts[j];
+    if constexpr (TABS)
+        for (int j = tid; j <= P.njobs; j += blockDim.x) s_tab_at[j] = P.tab_at[j];
     if (tid == 0) s_task[0] = (int)atomicAdd(P.task_ctr, 1ull);
     __syncthreads();
     auto find_job = [&](int t) {
@@ -202,6 +225,14 @@ __global__ void __launch_bounds__(kTileBatchThreads, 4)
             const unsigned d = (unsigned)__cvta_generic_to_shared(dstw + w);
             asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(srcw + w) : "memory");
         }
+        if constexpr (TABS) {
+            const int4 *src = P.tabs + s_tab_at[j];
+            int4 *dst = stabs + slot * P.tab_units;
+            for (int w = tid; w < s_tab_at[j + 1] - s_tab_at[j]; w += blockDim.x) {
+                const unsigned d = (unsigned)__cvta_generic_to_shared(dst + w);
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src + w) : "memory");
+            }
+        }
     };
     if (s_task[0] < P.total) {
         const int j = find_job(s_task[0]);
@@ -214,7 +245,7 @@ __global__ void __launch_bounds__(kTileBatchThreads, 4)
     for (int slot = 0;; slot ^= 1) {
         const int t = s_task[slot];
         if (t >= P.total) break;
-        const TilePass &a = s_job[slot].a;
+        const TileTask &a = s_job[slot].a;
         const int j = s_jobi[slot];
         // the next task's descriptor, under way during this tile
         const int tn = s_task[slot ^ 1];
@@ -236,9 +267,10 @@ __global__ void __launch_bounds__(kTileBatchThreads, 4)
             const int64_t base = tp_base(a, t - s_firsts[j]);
             E *out = static_cast<E *>(P.out[s_job[slot].transform]) + base;
             const E *src = s_job[slot].dep < 0 ? static_cast<const E *>(P.in[s_job[slot].transform]) + base : out;
-            constexpr int kOpt = kTpGlobalTw, kOne = kTpGlobalTw | kTpSingle;
-            const bool done = a.nst == 1 ? tp_run<ARITH, DIR, kOne>(a, sm, nullptr, emax, src, out)
-                                         : tp_run<ARITH, DIR, kOpt>(a, sm, nullptr, emax, src, out);
+            constexpr int kOpt = kTpChain | (TABS ? 0 : kTpGlobalTw), kOne = kOpt | kTpSingle;
+            const auto *tabs = TABS ? reinterpret_cast<const typename T::tw *>(stabs + slot * P.tab_units) : nullptr;
+            const bool done = a.nst == 1 ? tp_run<ARITH, DIR, kOne>(a, sm, tabs, emax, src, out)
+                                         : tp_run<ARITH, DIR, kOpt>(a, sm, tabs, emax, src, out);
             if (ARITH == kTpFixed && !done) {
                 double2 *smd = reinterpret_cast<double2 *>(smem_raw), *o = reinterpret_cast<double2 *>(out);
                 const double2 *i = reinterpret_cast<const double2 *>(src);
@@ -286,19 +318,32 @@ cudaError_t batch_setup(size_t smem, int threads, int *grid) {
     return cudaSuccess;
 }
 
-template <int ARITH, int DIR>
-cudaError_t tile_batch_setup(size_t smem, int *grid) {
+// What the tile batch needs of a launch: `grid` null to launch, else set it up.
+template <int ARITH, int DIR, bool TABS>
+cudaError_t tile_batch(const TileParams &P, size_t smem, int *grid, unsigned ctas, cudaStream_t st) {
+    if (!grid) {
+        tile_batch_kernel<ARITH, DIR, TABS><<<ctas, kTileBatchThreads, smem, st>>>(P);
+        return cudaGetLastError();
+    }
     if (smem > (size_t)kMaxDynSmem) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(tile_batch_kernel<ARITH, DIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(tile_batch_kernel<ARITH, DIR, TABS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kMaxDynSmem);
     int dev = 0, sms = 0, per_sm = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tile_batch_kernel<ARITH, DIR>, kTileBatchThreads, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tile_batch_kernel<ARITH, DIR, TABS>, kTileBatchThreads,
+                                                          smem);
     if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
     *grid = sms * per_sm;
     return e;
+}
+
+template <int ARITH>
+cudaError_t tile_batch_any(int dir, const TileParams &P, size_t smem, int *grid, unsigned ctas, cudaStream_t st) {
+    if (P.tab_units)
+        return dir < 0 ? tile_batch<ARITH, -1, true>(P, smem, grid, ctas, st) : tile_batch<ARITH, 1, true>(P, smem, grid, ctas, st);
+    return dir < 0 ? tile_batch<ARITH, -1, false>(P, smem, grid, ctas, st) : tile_batch<ARITH, 1, false>(P, smem, grid, ctas, st);
 }
 
 }  // namespace
@@ -309,10 +354,12 @@ struct Batch {
     size_t smem = 0;
     int njobs = 0;
     int64_t total = 0;
-    void *dev_mem = nullptr;  // jobs | firsts | task counter | done counters
+    void *dev_mem = nullptr;  // jobs | firsts | task counter | done counters | table places | tables
     BatchJob *jobs = nullptr;
     TileJob *tile_jobs = nullptr;  // set instead of jobs when every transform runs as tile passes
-    int emax_off = 0;
+    int emax_off = 0, tab_off = 0, tab_units = 0;  // tab_units 0: no tables
+    int *tab_at = nullptr;
+    int4 *tabs = nullptr;
     int64_t *firsts = nullptr;
     unsigned long long *task_ctr = nullptr;
     unsigned *done = nullptr;
@@ -362,7 +409,7 @@ fftu_status batch_create(int count, const fftu_handle *plans, Batch **out_batch)
                 TileJob J;
                 std::memset(&J, 0, sizeof(J));
                 J.transform = i;
-                J.a = views[i].whole[k];
+                fill_task(views[i].whole[k], J.a);
                 J.dep = last[i];
                 J.dep_tiles = last[i] < 0 ? 0 : tjobs[last[i]].a.tiles;
                 last[i] = (int)tjobs.size();
@@ -442,11 +489,20 @@ fftu_status batch_create(int count, const fftu_handle *plans, Batch **out_batch)
     b->njobs = (int)njobs;
     b->total = first;
     b->emax_off = (int)(tile_elems * esize);
-    b->smem = tiles ? tile_elems * esize + (b->is_double ? groups * sizeof(int) : 0) : max_tile_bytes;
+    std::vector<int> tab_at(1, 0);
+    for (const TileJob &J : tjobs) {
+        const int units = (int)((J.a.emax_off - J.a.tab_off + 15) / 16);
+        b->tab_units = std::max(b->tab_units, units);
+        tab_at.push_back(tab_at.back() + units);
+    }
+    if (b->tab_units > kTileBatchTable) b->tab_units = 0;
+    b->tab_off = (int)((b->emax_off + (b->is_double ? groups * sizeof(int) : 0) + 15) / 16 * 16);
+    b->smem = tiles ? b->tab_off + 2 * (size_t)b->tab_units * 16 : max_tile_bytes;
     b->threads = tiles ? kTileBatchThreads : std::min(kBatchThreads, (max_threads + 31) / 32 * 32);
     const size_t jb = (tiles ? sizeof(TileJob) : sizeof(BatchJob)) * njobs, fb = sizeof(int64_t) * njobs;
     b->counter_bytes = 16 + sizeof(unsigned) * njobs;
-    const size_t bytes = jb + fb + b->counter_bytes + 16;
+    const size_t tab_base = (jb + fb + b->counter_bytes + 16 + 15) / 16 * 16, tb = (sizeof(int) * tab_at.size() + 15) / 16 * 16;
+    const size_t bytes = tab_base + (b->tab_units ? tb + (size_t)tab_at.back() * 16 : 0);
     cudaError_t e = cudaMalloc(&b->dev_mem, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -461,6 +517,8 @@ fftu_status batch_create(int count, const fftu_handle *plans, Batch **out_batch)
     b->task_ctr = reinterpret_cast<unsigned long long *>(base + jb + fb);
     b->status = reinterpret_cast<int *>(base + jb + fb + 8);
     b->done = reinterpret_cast<unsigned *>(base + jb + fb + 16);
+    b->tab_at = reinterpret_cast<int *>(base + tab_base);
+    b->tabs = reinterpret_cast<int4 *>(base + tab_base + tb);
     // uploads on a private stream: creating a batch does not wait for transforms in flight
     cudaStream_t ps = nullptr;
     e = cudaStreamCreateWithFlags(&ps, cudaStreamNonBlocking);
@@ -468,15 +526,21 @@ fftu_status batch_create(int count, const fftu_handle *plans, Batch **out_batch)
                                              cudaMemcpyHostToDevice, ps);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->firsts, firsts.data(), fb, cudaMemcpyHostToDevice, ps);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->status, 0, sizeof(int), ps);
+    if (e == cudaSuccess && b->tab_units) {
+        e = cudaMemcpyAsync(b->tab_at, tab_at.data(), sizeof(int) * tab_at.size(), cudaMemcpyHostToDevice, ps);
+        if (e == cudaSuccess) {
+            if (b->is_double) tile_tables_kernel<kTpFixed><<<b->njobs, 128, 0, ps>>>(b->tile_jobs, b->tab_at, b->tabs);
+            else tile_tables_kernel<kTpF32><<<b->njobs, 128, 0, ps>>>(b->tile_jobs, b->tab_at, b->tabs);
+            e = cudaGetLastError();
+        }
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(ps);
     if (ps) cudaStreamDestroy(ps);
     if (e == cudaSuccess && tiles) {
-        if (b->is_double)
-            e = b->dir < 0 ? tile_batch_setup<kTpFixed, -1>(b->smem, &b->grid)
-                           : tile_batch_setup<kTpFixed, 1>(b->smem, &b->grid);
-        else
-            e = b->dir < 0 ? tile_batch_setup<kTpF32, -1>(b->smem, &b->grid)
-                           : tile_batch_setup<kTpF32, 1>(b->smem, &b->grid);
+        TileParams Q = {};
+        Q.tab_units = b->tab_units;
+        e = b->is_double ? tile_batch_any<kTpFixed>(b->dir, Q, b->smem, &b->grid, 0, nullptr)
+                         : tile_batch_any<kTpF32>(b->dir, Q, b->smem, &b->grid, 0, nullptr);
     } else if (e == cudaSuccess) {
         if (b->is_double)
             e = b->dir < 0 ? batch_setup<double2, -1>(b->smem, b->threads, &b->grid)
@@ -532,14 +596,13 @@ fftu_status batch_exec(Batch *b, const void *const *ins, void *const *outs, cuda
     int64_t grid = b->grid;
     if (grid > b->total) grid = b->total;
     if (b->tile_jobs) {
-        const unsigned g = (unsigned)grid;
-        if (b->is_double) {
-            if (b->dir < 0) tile_batch_kernel<kTpFixed, -1><<<g, b->threads, b->smem, st>>>(Q, b->emax_off);
-            else tile_batch_kernel<kTpFixed, 1><<<g, b->threads, b->smem, st>>>(Q, b->emax_off);
-        } else {
-            if (b->dir < 0) tile_batch_kernel<kTpF32, -1><<<g, b->threads, b->smem, st>>>(Q, b->emax_off);
-            else tile_batch_kernel<kTpF32, 1><<<g, b->threads, b->smem, st>>>(Q, b->emax_off);
-        }
+        Q.emax_off = b->emax_off;
+        Q.tab_off = b->tab_off;
+        Q.tab_units = b->tab_units;
+        Q.tab_at = b->tab_at;
+        Q.tabs = b->tabs;
+        e = b->is_double ? tile_batch_any<kTpFixed>(b->dir, Q, b->smem, nullptr, (unsigned)grid, st)
+                         : tile_batch_any<kTpF32>(b->dir, Q, b->smem, nullptr, (unsigned)grid, st);
     } else if (b->is_double) {
         if (b->dir < 0)
             batch_kernel<double2, -1><<<(unsigned)grid, b->threads, b->smem, st>>>(P);
@@ -551,7 +614,7 @@ fftu_status batch_exec(Batch *b, const void *const *ins, void *const *outs, cuda
         else
             batch_kernel<float2, 1><<<(unsigned)grid, b->threads, b->smem, st>>>(P);
     }
-    e = cudaGetLastError();
+    if (!b->tile_jobs) e = cudaGetLastError();
     if (e != cudaSuccess) {
         record_error("batch: kernel launch failed");
         return FFTU_ERR_CUDA;

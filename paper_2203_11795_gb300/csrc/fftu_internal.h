@@ -133,7 +133,7 @@ constexpr int kTpStages = 8, kTpFields = 8;
 struct BitField {
     int sh, mask, dst;  // ((x >> sh) & mask) << dst
 };
-struct TileStage {
+struct TileStageCore {
     int lg_r, pos;      // radix 2^lg_r on tile bits [pos, pos + lg_r)
     int tw_kind;        // 0: none; 1: w_{R T}^{r j} between the digits of an axis; 2: w_n^{k s} after the last digit of a
                         // phase-A axis
@@ -146,9 +146,12 @@ struct TileStage {
     int tab;            // the table's place in shared memory (elements): entry (r, q) at tab + (r << lg_q) + q
     const void *tw;     // w_n^e (complex128: in fixed point)
     const void *tw64;   // complex128: w_n^e as double2
+    int rb[5];          // shared slot of 1 << (pos + b)
+};
+struct TileStage : TileStageCore {
     int rx[32];         // shared slot of r << pos
 };
-struct TilePass {
+template <typename STAGE> struct TilePassOf {
     const void *src;
     void *dst;
     const void *mul;    // optional pointwise factor at the output's natural index
@@ -167,8 +170,10 @@ struct TilePass {
     int lg_scale;
     double scale;       // 2^lg_scale
     size_t tab_off, emax_off, smem;
-    TileStage st[kTpStages];
+    STAGE st[kTpStages];
 };
+using TilePass = TilePassOf<TileStage>;      // of a launch of one pass
+using TileTask = TilePassOf<TileStageCore>;  // of a batch, whose descriptors are copied to shared memory for each tile
 // Describe a pass over axes l0 .. l1 of the d-dimensional array n; p: phase A on that grid (NULL: whole axes); tw /
 // tw64: root tables per axis.  false: not served.
 bool make_tile_pass(int d, const int64_t *n, const int64_t *p, int l0, int l1, int is_double, int wide, int lg_v,

@@ -106,15 +106,15 @@ template <int ARITH, int DIR, int OPT>
 cudaError_t prepare_opt(const TilePass &a, int *per_sm) {
     cudaError_t e = cudaFuncSetAttribute(tile_pass_kernel<ARITH, DIR, OPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kMaxDynSmem);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || !per_sm) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, tile_pass_kernel<ARITH, DIR, OPT>, a.threads, a.smem);
 }
 
 template <int ARITH, int DIR>
 cudaError_t prepare_t(TilePass &a) {
-    int dev = 0, sms = 0, per_sm = 0, other = 0;
-    cudaError_t e = a.nst == 1 ? prepare_opt<ARITH, DIR, kTpMul | kTpSingle>(a, &other)
-                               : prepare_opt<ARITH, DIR, kTpMul>(a, &other);
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaError_t e = a.nst == 1 ? prepare_opt<ARITH, DIR, kTpMul | kTpSingle>(a, nullptr)
+                               : prepare_opt<ARITH, DIR, kTpMul>(a, nullptr);
     if (e == cudaSuccess)
         e = a.nst == 1 ? prepare_opt<ARITH, DIR, kTpSingle>(a, &per_sm) : prepare_opt<ARITH, DIR, 0>(a, &per_sm);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
@@ -252,8 +252,9 @@ bool make_tile_pass(int d, const int64_t *n, const int64_t *p, int l0, int l1, i
     // swizzle: the shifts that leave the lanes of one wavefront (16 of 8 bytes, 8 of 16) in distinct slots
     const int lw = is_double ? 3 : 4, m = (1 << lw) - 1;
     int best = 1 << 30;
-    for (int s1 = 1; s1 <= 13; ++s1)
-        for (int s2 = s1; s2 <= 13; ++s2) {
+    const int least = no > 2 ? 2 * no - 2 : no;  // every stage without conflicts
+    for (int s1 = 1; s1 <= 13 && best > least; ++s1)
+        for (int s2 = s1; s2 <= 13 && best > least; ++s2) {
             auto slot = [&](int e) { return (e ^ (e >> s1) ^ (s2 == s1 ? 0 : e >> s2)) & m; };
             int cost = 0;
             for (int si = 0; si < no; ++si) {
@@ -285,6 +286,7 @@ bool make_tile_pass(int d, const int64_t *n, const int64_t *p, int l0, int l1, i
         s.sh = si + 1 < no ? dg[order[si + 1]].bits : 0;
         s.tw = tw[l];
         s.tw64 = tw64[l];
+        for (int b = 0; b < g.bits; ++b) s.rb[b] = slot(1 << (g.pos + b));
         for (int r = 0; r < 1 << g.bits; ++r) s.rx[r] = slot(r << g.pos);
         const int lo_m = lo_of[l] + lg_p[l];  // lowest bit of m
         if (at + 1 < count_of[l]) {  // w_{R T}^{r j} = w_n^{r j n / (R T)}

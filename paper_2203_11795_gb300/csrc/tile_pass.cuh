@@ -28,6 +28,8 @@
 
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "fft_device.cuh"
 #include "fftu_internal.h"
 #include "fixed64.cuh"
@@ -36,16 +38,16 @@ namespace fftu {
 
 // ARITH of a tile pass; kTpF32w: complex64 with radix-32 stages (a kernel of its own, with twice the registers)
 constexpr int kTpF32 = 0, kTpFixed = 1, kTpF64 = 2, kTpF32w = 3;
-// OPT bits: the pointwise product in the last store; twiddles straight from the root tables (many kinds of pass in one
-// launch) instead of the stages' shared tables; a pass of one stage.
-constexpr int kTpMul = 1, kTpGlobalTw = 2, kTpSingle = 4;
+// OPT bits: the pointwise product in the last store; twiddles straight from the root tables instead of the stages' shared
+// tables; a pass of one stage; passes that follow one another in one launch (loads from L2).
+constexpr int kTpMul = 1, kTpGlobalTw = 2, kTpSingle = 4, kTpChain = 8;
 template <int ARITH> struct tp_type;
 template <> struct tp_type<kTpF32> { using elem = float2; using work = float2; using tw = float2; };
 template <> struct tp_type<kTpF32w> : tp_type<kTpF32> {};
 template <> struct tp_type<kTpFixed> { using elem = double2; using work = longlong2; using tw = int4; };
 template <> struct tp_type<kTpF64> { using elem = double2; using work = double2; using tw = double2; };
 
-template <int ARITH> __device__ __forceinline__ int tp_slot(const TilePass &a, int e) {
+template <int ARITH, typename P> __device__ __forceinline__ int tp_slot(const P &a, int e) {
     constexpr int m = sizeof(typename tp_type<ARITH>::elem) == 8 ? 15 : 7;
     return e ^ ((e >> a.swz[0]) & m) ^ ((e >> a.swz[1]) & m);
 }
@@ -68,28 +70,49 @@ template <int ARITH, int DIR, int R> __device__ __forceinline__ void tp_dft(type
     else dft_small<R, DIR>(v);
 }
 
-// Load of an input element.  In a launch whose passes follow one another (kTpGlobalTw) other SMs wrote it during the
-// kernel: from L2.
+// Load of an input element.  In a launch whose passes follow one another other SMs wrote it during the kernel: from L2.
 template <int OPT, typename E> __device__ __forceinline__ E tp_load(const E *p) {
-    if constexpr ((OPT & kTpGlobalTw) != 0) return __ldcg(p);
+    if constexpr ((OPT & kTpChain) != 0) return __ldcg(p);
     else return *p;
 }
+// Shared slots of the values of the fiber whose value 0 is at `slot`.  A launch of one pass has the XOR constants of all
+// values in the constant bank, an operand of the XOR.  A batch has its descriptors in shared memory: there a value's slot
+// is the slot of the value without its lowest bit, XOR that bit's constant (5 loads a stage instead of 32 or 64).
+template <typename STAGE, int R> struct TpSlots {
+    const STAGE &s;
+    int slot, at[std::is_same_v<STAGE, TileStage> ? 1 : R];
+    __device__ __forceinline__ TpSlots(const STAGE &s_, int slot_) : s(s_), slot(slot_) {
+        if constexpr (!std::is_same_v<STAGE, TileStage>) {
+            asm volatile("" : "+r"(slot));  // computed again for a stage's stores rather than kept in registers
+            at[0] = slot;
+        }
+    }
+    __device__ __forceinline__ int operator()(int r) {  // r ascending, known at compile time
+        if constexpr (std::is_same_v<STAGE, TileStage>) {
+            return slot ^ s.rx[r];
+        } else {
+            const int low = r & -r;
+            if (r) at[r] = at[r ^ low] ^ s.rb[low == 1 ? 0 : low == 2 ? 1 : low == 4 ? 2 : low == 8 ? 3 : 4];
+            return at[r];
+        }
+    }
+};
 // The column of stage s's twiddle table for the fiber at tile index e0.
-__device__ __forceinline__ int tp_column(const TileStage &s, int e0) {
+__device__ __forceinline__ int tp_column(const TileStageCore &s, int e0) {
     const int low = (e0 >> s.lo) & ((1 << (s.tw_kind == 1 ? s.lg_q : s.lg_p)) - 1);
     if (s.tw_kind == 1) return low;
     const int up = (e0 >> (s.pos + s.lg_r)) & ((1 << (s.lg_q - s.lg_p)) - 1);
     return low | (up << s.lg_p);
 }
 // Exponent of w_n for output digit r in column q.
-__device__ __forceinline__ unsigned tp_exponent(const TileStage &s, unsigned r, unsigned q) {
+__device__ __forceinline__ unsigned tp_exponent(const TileStageCore &s, unsigned r, unsigned q) {
     if (s.tw_kind == 1) return (r * q) << s.lg_step;
     const unsigned kp = tp_fields(s.k, s.nk, q >> s.lg_p);
     return (kp + (r << s.lg_step)) * (q & ((1u << s.lg_p) - 1));
 }
 // The twiddles of a stage on its fiber.
 template <int ARITH, int DIR, int OPT, int R>
-__device__ __forceinline__ void tp_twiddles(const TileStage &s, int e0, typename tp_type<ARITH>::work *v,
+__device__ __forceinline__ void tp_twiddles(const TileStageCore &s, int e0, typename tp_type<ARITH>::work *v,
                                             const typename tp_type<ARITH>::tw *tabs) {
     const int q = tp_column(s, e0);
     if constexpr (ARITH == kTpF64) {
@@ -111,8 +134,8 @@ __device__ __forceinline__ void tp_twiddles(const TileStage &s, int e0, typename
 
 // One stage of radix R.  FIRST: from src; LAST: to dst (both: a pass of one digit).  Returns false (kTpFixed, FIRST)
 // when the tile needs FP64 arithmetic.  `key` table: one magnitude key per v (kTpFixed).
-template <int ARITH, int DIR, int OPT, int R, bool FIRST, bool LAST>
-__device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_type<ARITH>::work *sm,
+template <int ARITH, int DIR, int OPT, int R, bool FIRST, bool LAST, typename P>
+__device__ __forceinline__ bool tp_stage(const P &a, int si, typename tp_type<ARITH>::work *sm,
                                          const typename tp_type<ARITH>::tw *tabs, int *emax,
                                          const typename tp_type<ARITH>::elem *src,
                                          typename tp_type<ARITH>::elem *dst) {
@@ -121,7 +144,7 @@ __device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_
     constexpr int RHO = lg_of<R>();
     int phi0 = threadIdx.x;
     asm volatile("" : "+r"(si), "+r"(phi0));  // per tile: nothing derived from them is kept in registers across tiles
-    const TileStage &s = a.st[si];
+    const auto &s = a.st[si];
     const int fibers = 1 << (a.lg_tile - RHO);
     // kTpFixed, FIRST: one fiber per thread at most (blockDim >= fibers), every thread at the barrier
     constexpr bool kOnce = ARITH == kTpFixed && FIRST;
@@ -173,8 +196,9 @@ __device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_
                 for (int r = 0; r < R; ++r) v[r] = tp_load<OPT>(p + ((size_t)r << a.in_bit));
             }
         } else {
+            TpSlots<std::remove_const_t<std::remove_reference_t<decltype(s)>>, R> at(s, slot);
 #pragma unroll
-            for (int r = 0; r < R; ++r) v[r] = sm[slot ^ s.rx[r]];
+            for (int r = 0; r < R; ++r) v[r] = sm[at(r)];
         }
         tp_dft<ARITH, DIR, R>(v);
         if constexpr (LAST) {
@@ -212,16 +236,17 @@ __device__ __forceinline__ bool tp_stage(const TilePass &a, int si, typename tp_
                     v[0] = fx_scale_down(v[0], s.sh);
                 }
             }
+            TpSlots<std::remove_const_t<std::remove_reference_t<decltype(s)>>, R> at(s, slot);
 #pragma unroll
-            for (int r = 0; r < R; ++r) sm[slot ^ s.rx[r]] = v[r];
+            for (int r = 0; r < R; ++r) sm[at(r)] = v[r];
         }
         if constexpr (kOnce) break;
     }
     return true;
 }
 
-template <int ARITH, int DIR, int OPT, bool FIRST, bool LAST>
-__device__ __forceinline__ bool tp_stage_any(const TilePass &a, int si, typename tp_type<ARITH>::work *sm,
+template <int ARITH, int DIR, int OPT, bool FIRST, bool LAST, typename P>
+__device__ __forceinline__ bool tp_stage_any(const P &a, int si, typename tp_type<ARITH>::work *sm,
                                              const typename tp_type<ARITH>::tw *tabs, int *emax,
                                              const typename tp_type<ARITH>::elem *src,
                                              typename tp_type<ARITH>::elem *dst) {
@@ -242,11 +267,11 @@ __device__ __forceinline__ bool tp_stage_any(const TilePass &a, int si, typename
 }
 
 // Twiddle tables of the stages (F32 / Fixed).
-template <int ARITH>
-__device__ __forceinline__ void tp_tables(const TilePass &a, typename tp_type<ARITH>::tw *tabs) {
+template <int ARITH, typename P>
+__device__ __forceinline__ void tp_tables(const P &a, typename tp_type<ARITH>::tw *tabs) {
     using TW = typename tp_type<ARITH>::tw;
     for (int si = 0; si < a.nst; ++si) {
-        const TileStage &s = a.st[si];
+        const auto &s = a.st[si];
         if (s.tw_kind == 0) continue;
         const TW *tw = static_cast<const TW *>(s.tw);
         const int n = 1 << (s.lg_r + s.lg_q);
@@ -258,8 +283,8 @@ __device__ __forceinline__ void tp_tables(const TilePass &a, typename tp_type<AR
     }
 }
 
-template <int ARITH, int DIR, int OPT>
-__device__ __forceinline__ bool tp_run(const TilePass &a, typename tp_type<ARITH>::work *sm,
+template <int ARITH, int DIR, int OPT, typename P>
+__device__ __forceinline__ bool tp_run(const P &a, typename tp_type<ARITH>::work *sm,
                                        const typename tp_type<ARITH>::tw *tabs, int *emax,
                                        const typename tp_type<ARITH>::elem *src, typename tp_type<ARITH>::elem *dst) {
     if constexpr ((OPT & kTpSingle) != 0) return tp_stage_any<ARITH, DIR, OPT, true, true>(a, 0, sm, tabs, emax, src, dst);
@@ -273,13 +298,13 @@ __device__ __forceinline__ bool tp_run(const TilePass &a, typename tp_type<ARITH
     return true;
 }
 
-template <int DIR, int OPT>
-__device__ __noinline__ void tp_run_fp64(const TilePass &a, double2 *sm, const double2 *src, double2 *dst) {
+template <int DIR, int OPT, typename P>
+__device__ __noinline__ void tp_run_fp64(const P &a, double2 *sm, const double2 *src, double2 *dst) {
     tp_run<kTpF64, DIR, OPT>(a, sm, nullptr, nullptr, src, dst);
 }
 
 // Element offset of tile t.
-__device__ __forceinline__ int64_t tp_base(const TilePass &a, int64_t t) {
+template <typename P> __device__ __forceinline__ int64_t tp_base(const P &a, int64_t t) {
     if (a.lg_inner < 0) return t << a.lg_tile;
     const int lg_c = a.lg_inner - a.lg_v;  // tiles along the inner positions
     return ((t >> lg_c) << (a.lg_g + a.lg_inner)) + ((t & (((int64_t)1 << lg_c) - 1)) << a.lg_v);

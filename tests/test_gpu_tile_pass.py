@@ -138,3 +138,43 @@ def test_batch_of_tile_passes(fftu, dt, inplace):
         p.close()
     for x, o, s in zip(xs, outs, scale):
         assert oracle.rel_l2(o.cpu().numpy() * s, oracle.fftn(x.astype(np.complex128) * s)) <= tol(dt, x.size)
+
+
+@pytest.mark.parametrize("dt", [np.complex64, np.complex128])
+@pytest.mark.parametrize("longest", [512, 1024], ids=lambda n: f"longest{n}")
+def test_batch_tables(fftu, dt, longest):
+    """Batches on both sides of the twiddle tables' largest size (512-point complex64 axes have them, 1024-point ones and
+    512-point complex128 ones take the roots), with passes of one to three stages and without twiddles."""
+    import torch
+    shapes = [(longest, 4), (2, longest), (8, 8, 8), (16, 16, 16), (64, 32, 128), (256, 64), (2,)]
+    xs = [complex_uniform(810 + i, s, dtype=dt) for i, s in enumerate(shapes)]
+    ts = [torch.from_numpy(x).cuda() for x in xs]
+    outs = [torch.empty_like(t) for t in ts]
+    plans = [fftu.Plan(s, None, dtype=t.dtype, inverse=True) for s, t in zip(shapes, ts)]
+    b = fftu.fftu_batch_create([p.handle for p in plans])
+    for _ in range(2):
+        fftu.fftu_batch_exec(b, [t.data_ptr() for t in ts], [o.data_ptr() for o in outs],
+                             torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    fftu.fftu_batch_check_status(b)
+    fftu.fftu_batch_destroy(b)
+    for p in plans:
+        p.close()
+    for x, o in zip(xs, outs):
+        assert oracle.rel_l2(o.cpu().numpy(), oracle.fftn(x.astype(np.complex128), inverse=True)) <= tol(dt, x.size)
+
+
+@pytest.mark.parametrize("shape", [(512, 64, 64), (8, 64, 64, 64)], ids=shape_id)
+def test_two_axes_of_64_complex128(fftu, shape):
+    """Contiguous planes of 64 x 64 in one tile, in and out of place; one plane takes FP64 arithmetic."""
+    import torch
+    x = complex_uniform(820, shape, dtype=np.complex128)
+    x[1] *= 2.0 ** -980
+    t = torch.from_numpy(x).cuda()
+    with fftu.Plan(shape, None, dtype=t.dtype) as plan:
+        y = plan.exec(t)
+        assert torch.equal(t, torch.from_numpy(x).cuda())
+        plan.exec(t, t)
+        assert torch.equal(t, y)
+        plan.check_device_status()
+    assert oracle.rel_l2(y.cpu().numpy(), oracle.fftn(x)) <= tol(np.complex128, x.size)
