@@ -1,6 +1,7 @@
 // Tile passes (tile_pass.cuh): kernel, launch, and the planner that splits a pass into stages.
 #include <cuda_runtime.h>
 
+#include <climits>
 #include <cstring>
 #include <utility>
 
@@ -11,7 +12,7 @@
 namespace fftu {
 namespace {
 
-// Persistent: the twiddle tables are built once per CTA.  64 registers (1024 threads per SM, in CTAs of 256 for the usual
+// Grid: prepare_t.  The twiddle tables are built once per CTA.  64 registers (1024 threads per SM, in CTAs of 256 for the usual
 // tiles), 128 with radix-32 stages.
 template <int ARITH, int DIR, int OPT>
 __global__ void __launch_bounds__(ARITH == kTpF32w ? 512 : 1024) tile_pass_kernel(const __grid_constant__ TilePass a) {
@@ -120,7 +121,13 @@ cudaError_t prepare_t(TilePass &a) {
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
-    a.grid = sms * per_sm;
+    // Persistent CTAs, which build their tables once, where these are a sizeable part of a tile; otherwise a CTA per tile:
+    // the SMs take the tiles in order as they come free, so that the last wave is short and neighbouring tiles stay close
+    // in time.  Persistent against a CTA per tile: complex128 64^4 599 and 534 us, 128^3 94 and 81, 256 x 16 x 16 x 256 696
+    // and 631 (tables of up to a seventh of the tile), 2048^2 202 and 206; complex64 32^5 335 and 322 (a 64th), 256^3 134.5
+    // and 135.8 (a 16th), 1024 x 4096 37 and 41, 256 x 256 x 128 on 8^3 89 and 95.
+    const size_t tables = a.emax_off - a.tab_off, tile = (size_t)(ARITH == kTpFixed ? 16 : 8) << a.lg_tile;
+    a.grid = tables * (ARITH == kTpFixed ? 7 : 32) <= tile ? INT_MAX : sms * per_sm;
     return e;
 }
 
