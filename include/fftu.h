@@ -81,7 +81,8 @@ typedef enum {
 } fftu_schedule;
 
 /* Arithmetic of the radix-16 DFT stages of the strided passes (complex64 plans only).
- * NATIVE: FP32 (complex64) or FP64 (complex128) on the CUDA cores.
+ * NATIVE: FP32 (complex64), or 64-bit fixed point with FP64 where values cannot be scaled (complex128),
+ * on the CUDA cores.
  * SPLIT_BF16 / SPLIT_FP16: each radix-16 stage of 8 butterflies is a real 32 x 32 contraction on
  * the tensor cores (mma.sync m16n8k16, FP32 accumulation) with both operands split into a 16-bit
  * high and low part (three products; the low x low term is dropped); FP16 operands are scaled per
@@ -328,8 +329,8 @@ fftu_status fftu_selftest_bounded_wait(double limit_s, double *waited_s);
 /* Measurement helper (not part of the method): the sustained FP64 fused multiply-add rate of the
  * current device in GFLOP/s (2 flops per FMA), from a kernel that keeps every SM's FP64 pipe busy with
  * independent FMA chains, timed with CUDA events; best of `reps` (1..100) timed launches after one
- * warm-up.  complex128 transforms are bound by this rate rather than by HBM bandwidth on GB300, so
- * their roofline is stated against it.  Allocates and frees 8 bytes of device memory and a stream;
+ * warm-up.  complex128 transforms run their DFT stages in 64-bit fixed point on the integer units,
+ * past this rate.  Allocates and frees 8 bytes of device memory and a stream;
  * synchronises that stream.  FFTU_ERR_ARG for a NULL gflops or reps out of range. */
 fftu_status fftu_measure_fp64_rate(int reps, double *gflops);
 
