@@ -1,7 +1,7 @@
 // Tile passes (tile_pass.cuh): kernel, launch, and the planner that splits a pass into stages.
 #include <cuda_runtime.h>
 
-#include <climits>
+#include <algorithm>
 #include <cstring>
 #include <utility>
 
@@ -27,7 +27,10 @@ __global__ void __launch_bounds__(ARITH == kTpF32w ? 512 : 1024) tile_pass_kerne
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     tp_tables<ARITH>(a, tabs);  // plan data, not written by earlier kernels
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    for (int64_t t = blockIdx.x; t < a.tiles; t += gridDim.x) {
+    // a.chunk tiles in a row, or (0) every gridDim.x-th tile
+    const int64_t step = a.chunk ? 1 : gridDim.x, first = a.chunk ? blockIdx.x * (int64_t)a.chunk : blockIdx.x;
+    const int64_t end = a.chunk && first + a.chunk < a.tiles ? first + a.chunk : a.tiles;
+    for (int64_t t = first; t < end; t += step) {
         __syncthreads();  // tables ready; the previous tile's last stage done with its slots and exponents
         if constexpr (ARITH == kTpFixed) {
             for (int i = threadIdx.x; i < 1 << a.lg_groups; i += blockDim.x) emax[i] = 0;
@@ -83,13 +86,12 @@ int gf2_rank(int *v, int n) {
 
 template <int ARITH, int DIR>
 cudaError_t launch_t(const TilePass &a, cudaStream_t st) {
-    int64_t grid = a.tiles < a.grid ? a.tiles : a.grid;
     // programmatic launch: the CTAs may start, and build their tables, while the kernel before this one finishes
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = dim3((unsigned)a.grid);
     cfg.blockDim = dim3((unsigned)a.threads);
     cfg.dynamicSmemBytes = a.smem;
     cfg.stream = st;
@@ -121,13 +123,20 @@ cudaError_t prepare_t(TilePass &a) {
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
-    // Persistent CTAs, which build their tables once, where these are a sizeable part of a tile; otherwise a CTA per tile:
-    // the SMs take the tiles in order as they come free, so that the last wave is short and neighbouring tiles stay close
-    // in time.  Persistent against a CTA per tile: complex128 64^4 599 and 534 us, 128^3 94 and 81, 256 x 16 x 16 x 256 696
-    // and 631 (tables of up to a seventh of the tile), 2048^2 202 and 206; complex64 32^5 335 and 322 (a 64th), 256^3 134.5
-    // and 135.8 (a 16th), 1024 x 4096 37 and 41, 256 x 256 x 128 on 8^3 89 and 95.
+    // The twiddle tables are built once per CTA.  Where they are a small part of a tile, a CTA per tile: the SMs take the
+    // tiles in order as they come free, so that the last wave is short and neighbouring tiles stay close in time.
+    // Persistent against a CTA per tile: complex128 64^4 599 and 534 us, 128^3 94 and 81, 256 x 16 x 16 x 256 696 and 631
+    // (tables of up to a seventh of the tile), 2048^2 202 and 206; complex64 32^5 335 and 322 (a 64th), 256^3 134.5 and
+    // 135.8 (a 16th), 1024 x 4096 37 and 41, 256 x 256 x 128 on 8^3 89 and 95.  With larger tables, a few tiles in a row per
+    // CTA, for as many as keep that proportion, in complex128 and on long complex64 axes: 512 x 512 x 64 complex128
+    // persistent 620 and 595, 64 x 1024 x 1024 complex64 638 and 597; not on shorter complex64 axes (512 x 64 x 512 146 and
+    // 151) or where they would be fewer CTAs than fit at once.
     const size_t tables = a.emax_off - a.tab_off, tile = (size_t)(ARITH == kTpFixed ? 16 : 8) << a.lg_tile;
-    a.grid = tables * (ARITH == kTpFixed ? 7 : 32) <= tile ? INT_MAX : sms * per_sm;
+    const int64_t resident = (int64_t)sms * per_sm;
+    const int64_t c = std::max<int64_t>(1, (tables * (ARITH == kTpFixed ? 7 : 32) + tile - 1) / tile);
+    const bool rows = ARITH == kTpFixed || (ARITH == kTpF32w && a.lg_g >= 10);
+    a.chunk = c == 1 || (rows && c * resident <= a.tiles) ? (int)c : 0;
+    a.grid = a.chunk ? (int)((a.tiles + c - 1) / c) : (int)std::min(a.tiles, resident);
     return e;
 }
 
