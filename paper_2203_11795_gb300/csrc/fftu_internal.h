@@ -158,6 +158,7 @@ template <typename STAGE> struct TilePassOf {
     int64_t tiles;
     int grid, threads;
     int chunk;          // consecutive tiles of a CTA; 0: every grid-th tile
+    int resident;       // CTAs that fit at once
     int wide;           // complex64: radix-32 stages
     int once;           // one stage, one fiber per thread, a barrier between the loads and the stores
     int lg_g, lg_v, lg_inner, lg_tile;  // lg_g: positions of the axes; lg_inner < 0: contiguous

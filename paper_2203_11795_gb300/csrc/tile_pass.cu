@@ -132,7 +132,7 @@ cudaError_t prepare_t(TilePass &a) {
     // persistent 620 and 595, 64 x 1024 x 1024 complex64 638 and 597; not on shorter complex64 axes (512 x 64 x 512 146 and
     // 151) or where they would be fewer CTAs than fit at once.
     const size_t tables = a.emax_off - a.tab_off, tile = (size_t)(ARITH == kTpFixed ? 16 : 8) << a.lg_tile;
-    const int64_t resident = (int64_t)sms * per_sm;
+    const int64_t resident = a.resident = sms * per_sm;
     const int64_t c = std::max<int64_t>(1, (tables * (ARITH == kTpFixed ? 7 : 32) + tile - 1) / tile);
     const bool rows = ARITH == kTpFixed || (ARITH == kTpF32w && a.lg_g >= 10);
     a.chunk = c == 1 || (rows && c * resident <= a.tiles) ? (int)c : 0;
