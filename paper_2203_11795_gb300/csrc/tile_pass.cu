@@ -130,12 +130,12 @@ cudaError_t prepare_t(TilePass &a) {
     // 135.8 (a 16th), 1024 x 4096 37 and 41, 256 x 256 x 128 on 8^3 89 and 95.  With larger tables, a few tiles in a row per
     // CTA, for as many as keep that proportion, in complex128 and on long complex64 axes: 512 x 512 x 64 complex128
     // persistent 620 and 595, 64 x 1024 x 1024 complex64 638 and 597; not on shorter complex64 axes (512 x 64 x 512 146 and
-    // 151) or where they would be fewer CTAs than fit at once.
+    // 151), for fewer than four waves of them (32 x 1024 x 1024 286 and 293) or one of complex128 (2048^2 202 and 201).
     const size_t tables = a.emax_off - a.tab_off, tile = (size_t)(ARITH == kTpFixed ? 16 : 8) << a.lg_tile;
     const int64_t resident = a.resident = sms * per_sm;
     const int64_t c = std::max<int64_t>(1, (tables * (ARITH == kTpFixed ? 7 : 32) + tile - 1) / tile);
     const bool rows = ARITH == kTpFixed || (ARITH == kTpF32w && a.lg_g >= 10);
-    a.chunk = c == 1 || (rows && c * resident <= a.tiles) ? (int)c : 0;
+    a.chunk = c == 1 || (rows && (ARITH == kTpFixed ? 1 : 4) * c * resident <= a.tiles) ? (int)c : 0;
     a.grid = a.chunk ? (int)((a.tiles + c - 1) / c) : (int)std::min(a.tiles, resident);
     return e;
 }
