@@ -17,6 +17,8 @@
 // outputs (b div Ns) Ns R + (b mod Ns) + r Ns.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "fft_device.cuh"
 #include "fftu_internal.h"
 #include "generic_tiles.cuh"
@@ -48,7 +50,7 @@ __global__ void __launch_bounds__(kAxisThreads) axis_pass_kernel(const __grid_co
     }
 }
 
-// complex128: the stages in fixed point (axis_tile_fx), the columns' exponents after the tile.
+// complex128: the stages in fixed point (axis_tile_fx), the columns' exponents and sizes after the tile.
 template <int DIR, int R0>
 __global__ void __launch_bounds__(kAxisThreads) axis_fixed_kernel(const __grid_constant__ AxisPass a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -179,8 +181,8 @@ cudaError_t prepare_axis_t() {
 size_t axis_pass_smem_bytes(const AxisPass &a, int is_double) {
     const size_t tile = (size_t)a.tile * (is_double ? sizeof(double2) : sizeof(float2));
     if (!is_double && (a.tc == 1 || a.tc == 2)) return (tile + 127) / 128 * 128 + umma_smem_bytes(a.threads);
-    // complex128: one exponent per column (tile / len) after the tile
-    return is_double ? tile + sizeof(int) * (size_t)(a.tile / a.len) : tile;
+    // complex128: one exponent per column (tile / len) after the tile, then the sizes that the stages leave
+    return is_double ? tile + std::max(a.nstages, 1) * sizeof(int) * (size_t)(a.tile / a.len) : tile;
 }
 
 cudaError_t launch_fixed_table(void *dst, const void *src, int64_t n, cudaStream_t st) {

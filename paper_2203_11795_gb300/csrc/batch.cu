@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(kTileBatchThreads, 4) tile_batch_kernel(const 
             s_ok = dep < 0 || wait_counter_geq(P.done + dep, (unsigned)s_job[slot].dep_tiles, P.spin_limit_ns, P.status);
         }
         if constexpr (ARITH == kTpFixed)
-            for (int i = tid; i < 1 << a.lg_groups; i += blockDim.x) emax[i] = 0;
+            for (int i = tid; i < tp_entries(a); i += blockDim.x) emax[i] = 0;
         __syncthreads();
         int claimed = 0;
         if (tid == 0 && tn < P.total) claimed = (int)atomicAdd(P.task_ctr, 1ull);  // used after the tile
@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(kTileBatchThreads, 4) tile_batch_kernel(const 
             const int64_t base = tp_base(a, t - s_firsts[j]);
             E *out = static_cast<E *>(P.out[s_job[slot].transform]) + base;
             const E *src = s_job[slot].dep < 0 ? static_cast<const E *>(P.in[s_job[slot].transform]) + base : out;
-            constexpr int kOpt = kTpChain | (TABS ? 0 : kTpGlobalTw), kOne = kOpt | kTpSingle;
+            constexpr int kOpt = kTpChain | kTpShifts | (TABS ? 0 : kTpGlobalTw), kOne = kOpt | kTpSingle;
             const auto *tabs = TABS ? reinterpret_cast<const typename T::tw *>(stabs + slot * P.tab_units) : nullptr;
             const bool done = a.nst == 1 ? tp_run<ARITH, DIR, kOne>(a, sm, tabs, emax, src, out)
                                          : tp_run<ARITH, DIR, kOpt>(a, sm, tabs, emax, src, out);
@@ -415,7 +415,7 @@ fftu_status batch_create(int count, const fftu_handle *plans, Batch **out_batch)
                 last[i] = (int)tjobs.size();
                 tjobs.push_back(J);
                 tile_elems = std::max(tile_elems, (size_t)1 << J.a.lg_tile);
-                groups = std::max(groups, (size_t)1 << J.a.lg_groups);
+                groups = std::max(groups, (size_t)tp_entries(J.a));
             }
     }
     std::vector<BatchJob> jobs;

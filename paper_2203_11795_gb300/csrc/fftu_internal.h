@@ -140,12 +140,16 @@ struct TileStageCore {
     int lo, lg_q;       // twiddle column q in [2^lg_q]: kind 1 j = tile bits [lo, lo + lg_q); kind 2 class s = tile bits
                         // [lo, lo + lg_p) and the axis' bits above the digit
     int lg_p, lg_step;  // kind 1: exponent r j 2^lg_step; kind 2: exponent (k_prev + r 2^lg_step) s
-    int sh;             // complex128: log2 of the next stage's points (its values are scaled down by them)
     int nk;             // kind 2: k_prev = fields k[] of the bits above the digit
     BitField k[2];
     int tab;            // the table's place in shared memory (elements): entry (r, q) at tab + (r << lg_q) + q
     const void *tw;     // w_n^e (complex128: in fixed point)
     const void *tw64;   // complex128: w_n^e as double2
+    // complex128 (fixed64.cuh)
+    int sh, pre;        // shifts for any data: of the stage's results, through its twiddles, and of its inputs
+    int size_in;        // shift of its inputs by the groups' sizes in entries size_in (0: none)
+    int size_out;       // where it leaves its results' sizes for the next stage
+    int warp;           // the fibers of a warp are of one exponent group
     int rb[5];          // shared slot of 1 << (pos + b)
 };
 struct TileStage : TileStageCore {
@@ -169,6 +173,10 @@ template <typename STAGE> struct TilePassOf {
     BitField last[kTpFields], out[kTpFields];  // last stage: thread index -> tile index, -> element offset
     BitField group[kTpFields];                 // complex128: tile index -> exponent group (one per sub-DFT)
     int lg_groups;
+    int shifts;                                // complex128: some stage shifts its inputs (pre, size_in)
+    int sizes;                                 // stages that do it by their groups' sizes: entries 1 .. sizes,
+    int size_lg[kTpStages], size_room[kTpStages];  // log2 of the stage's points, room that it leaves
+    int shift;                                 // sum of the stages' sh and pre
     int lg_scale;
     double scale;       // 2^lg_scale
     size_t tab_off, emax_off, smem;

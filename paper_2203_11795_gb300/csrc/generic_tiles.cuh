@@ -333,13 +333,14 @@ __device__ __forceinline__ void axis_tile(const AxisPass &a, int64_t t, C *sm, c
 
 // ---- complex128 strided pass in fixed point (fixed64.cuh) -----------------------------------------
 // The tile's slots hold double2 as loaded, then longlong2 (both 16 bytes) from the first stage on.  One
-// exponent per sub-FFT (class and vector): emax[column] is the largest key of its inputs.
+// exponent per sub-FFT (class and vector): emax[column] is the largest key of its inputs, emax[i columns + column]
+// the size (fx_size) that stage i - 1 leaves.
 
 // A Stockham stage on the fixed-point tile (the index maps of stockham_stage).  FIRST: reads double2, finds the
-// columns' exponents; returns false, the tile unchanged, when some value needs FP64 arithmetic.
+// columns' exponents; returns false, the tile unchanged, when some value needs FP64 arithmetic.  si: the stage's number.
 template <int DIR, int R, bool FIRST>
 __device__ __forceinline__ bool fx_stage(longlong2 *sm, const int4 *__restrict__ tw, const AxisPass &a, int Ns,
-                                         int *emax, int tid, int nthreads) {
+                                         int si, int *emax, int tid, int nthreads) {
     constexpr int B = 8 / R;  // butterflies per thread
     constexpr int RHO = lg_of<R>();
     const int lg_cols = a.lg_Gt + a.lg_V;
@@ -349,6 +350,7 @@ __device__ __forceinline__ bool fx_stage(longlong2 *sm, const int4 *__restrict__
     const int twstep = a.nl / (Ns * R);
     const int lg_ns = 31 - __clz(Ns);
     longlong2 v[B][R];
+    [[maybe_unused]] int own[B];  // FIRST: the butterflies' own keys
     int bad = 0;
 #pragma unroll
     for (int q = 0; q < B; ++q) {
@@ -358,29 +360,26 @@ __device__ __forceinline__ bool fx_stage(longlong2 *sm, const int4 *__restrict__
             const int base = a.contiguous ? ((col >> a.lg_Gt) << a.lg_nlt) + (col & (a.Gt - 1)) : col;
             const int js = a.contiguous ? a.Gt : cols;
             if constexpr (FIRST) {
-                int key = 0;
+                double2 x[R];
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     v[q][r] = sm[smi(base + (b + r * per_col) * js, a.swz)];
-                    const int k = fx_key(fx_bits(v[q][r]));
-                    key = k > key ? k : key;
+                    x[r] = fx_bits(v[q][r]);
                 }
-                unsigned lo = 0;
-                if (key == 0) {
-#pragma unroll
-                    for (int r = 0; r < R; ++r) lo |= (unsigned)v[q][r].x | (unsigned)v[q][r].y;
-                }
-                if (!fx_plain(key, lo)) bad = 1;
-                atomicMax(emax + col, key);
+                own[q] = fx_keys<R>(x);
+                if (!fx_plain(own[q])) bad = 1;
+                atomicMax(emax + col, own[q]);
             } else {
                 const int k = b & (Ns - 1);
+                const int sh = fx_shift(emax[si * cols + col], RHO, kFxRoomProduct);
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
-                    longlong2 x = fx_scale_down(sm[smi(base + (b + r * per_col) * js, a.swz)], RHO);
-                    if (r > 0) x = fx_cmul<DIR>(x, tw[r * k * twstep]);
-                    v[q][r] = x;
+                    v[q][r] = sm[smi(base + (b + r * per_col) * js, a.swz)];
+                    if (r > 0) v[q][r] = fx_cmul<DIR>(v[q][r], tw[r * k * twstep]);
                 }
+                fx_floor<R>(v[q], sh);
                 fx_dft<R, DIR>(v[q]);
+                fx_mend<R>(v[q], sh);
             }
         }
     }
@@ -397,14 +396,24 @@ __device__ __forceinline__ bool fx_stage(longlong2 *sm, const int4 *__restrict__
             const int base = a.contiguous ? ((col >> a.lg_Gt) << a.lg_nlt) + (col & (a.Gt - 1)) : col;
             const int js = a.contiguous ? a.Gt : cols;
             if constexpr (FIRST) {
-                const int E = fx_exp(emax[col]);
+                const int key = emax[col];
+                const bool fine = fx_fine(own[q], key);
+                const int E = fx_exp(key) - (fine ? kFxFine : 0);
+                double2 x[R];
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const double2 x = fx_bits(v[q][r]);
-                    v[q][r] = mk<longlong2>(fx_in<kFxTop - RHO>(x.x, E), fx_in<kFxTop - RHO>(x.y, E));
-                }
+                for (int r = 0; r < R; ++r) x[r] = fx_bits(v[q][r]);
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    v[q][r] = mk<longlong2>(fx_in<kFxTop - RHO>(x[r].x, E), fx_in<kFxTop - RHO>(x[r].y, E));
                 fx_dft<R, DIR>(v[q]);
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[q][r] = fx_scale_down(v[q][r], 1);  // for the products
+                if (fine) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) v[q][r] = fx_scale_down(v[q][r], kFxFine);
+                }
             }
+            if (si + 1 < a.nstages) atomicMax(emax + (si + 1) * cols + col, fx_size<R>(v[q]));
             const int k = b & (Ns - 1);
             const int o = ((b >> lg_ns) << lg_ns) * R + k;
 #pragma unroll
@@ -422,25 +431,36 @@ __device__ __noinline__ void axis_finish_fp64(const AxisPass &a, const AxisOrigi
     axis_finish<double2, DIR, R0>(a, o, sm, dst, tw);
 }
 
-// One complex128 tile of a strided pass.  emax: one int per column (tile / len), in shared memory.
+// One complex128 tile of a strided pass.  emax: an int per column (tile / len) and stage, in shared memory.
 template <int DIR, int R0>
 __device__ __forceinline__ void axis_tile_fx(const AxisPass &a, int64_t t, double2 *sm, int *emax,
                                              const double2 *__restrict__ src, double2 *__restrict__ dst) {
-    const int tid = threadIdx.x, nt = blockDim.x;
+    int tid = threadIdx.x;
+    asm volatile("" : "+r"(tid));  // per tile: nothing derived from it is kept in registers across tiles
+    const int nt = blockDim.x;
     const AxisOrigin o = axis_origin(a, t);
-    for (int i = tid; i < 1 << (a.lg_Gt + a.lg_V); i += nt) emax[i] = 0;
+    const int cols = 1 << (a.lg_Gt + a.lg_V);
+    for (int i = tid; i < max(a.nstages, 1) * cols; i += nt) emax[i] = 0;
     axis_load<double2>(a, o, sm, src);
     longlong2 *fx = reinterpret_cast<longlong2 *>(sm);
     const int4 *__restrict__ tw = static_cast<const int4 *>(a.twf);
-    int Ns = R0 > 1 ? R0 : 8;
+    constexpr int kFirst = R0 > 1 ? R0 : 8;
     // len = 1 (every p_l = 1): a copy with scale
-    if (a.len == 1 || !fx_stage<DIR, (R0 > 1 ? R0 : 8), true>(fx, tw, a, 1, emax, tid, nt)) {
+    if (a.len == 1 || !fx_stage<DIR, kFirst, true>(fx, tw, a, 1, 0, emax, tid, nt)) {
         axis_finish_fp64<DIR, R0>(a, o, sm, dst, static_cast<const double2 *>(a.tw));
         return;
     }
-    for (; Ns < a.len; Ns *= 8) fx_stage<DIR, 8, false>(fx, tw, a, Ns, emax, tid, nt);
-    // 1/N is a power of two and goes into the exponent
+    for (int Ns = kFirst, si = 1; Ns < a.len; Ns *= 8, ++si) fx_stage<DIR, 8, false>(fx, tw, a, Ns, si, emax, tid, nt);
+    // the columns' exponents; 1/N is a power of two and goes into them
     const int lg_scale = (__double2hiint(a.scale) >> 20) - 1023;
+    for (int c = tid; c < cols; c += nt) {
+        const int key = emax[c];
+        int shift = 1;
+        for (int i = 1; i < a.nstages; ++i) shift += fx_shift(emax[i * cols + c], 3, kFxRoomProduct);
+        const int e0 = fx_out_exp(fx_exp(key), lg_of<kFirst>(), shift) + lg_scale;
+        emax[c] = e0;
+    }
+    __syncthreads();
     for (int e = tid; e < a.tile; e += nt) {
         int lpo, v;
         if (a.contiguous) {
@@ -466,9 +486,8 @@ __device__ __forceinline__ void axis_tile_fx(const AxisPass &a, int64_t t, doubl
             x = fx[smi(e, a.swz)];
             gp = o.c0 + cl + ((int64_t)(lpo >> a.lg_Gt) << a.lg_G);
         }
-        const int key = emax[a.contiguous ? (v << a.lg_Gt) + cl : (cl << a.lg_V) + v];
-        if (key == 0) x = mk<longlong2>(0, 0);  // all zeros: no trace of the products' rounding constants
-        const int e0 = fx_out_exp(fx_exp(key), a.lg_len) + lg_scale;
+        const int col = a.contiguous ? (v << a.lg_Gt) + cl : (cl << a.lg_V) + v;
+        const int e0 = emax[col];
         const int64_t g = a.contiguous ? o.gbase + (int64_t)v * a.nl + gp : o.gbase + gp * a.inner + v;
         dst[g] = mk<double2>(fx_out(x.x, e0), fx_out(x.y, e0));
     }
@@ -494,18 +513,8 @@ template <int DIR, int LO, int HI> __device__ __noinline__ void fiber_fp64(doubl
 template <int DIR, int LO, int HI> __device__ __forceinline__ void fiber_dft(double2 *v, int lg_scale) {
     constexpr int PG = LO * HI;
     constexpr int RHO = lg_of<PG>();
-    int key = 0;
-#pragma unroll
-    for (int j = 0; j < PG; ++j) {
-        const int k = fx_key(v[j]);
-        key = k > key ? k : key;
-    }
-    unsigned lo = 0;
-    if (key == 0) {
-#pragma unroll
-        for (int j = 0; j < PG; ++j) lo |= (unsigned)__double2loint(v[j].x) | (unsigned)__double2loint(v[j].y);
-    }
-    if (!fx_plain(key, lo)) {
+    const int key = fx_keys<PG>(v);
+    if (!fx_plain(key)) {
         double2 c[PG];
 #pragma unroll
         for (int j = 0; j < PG; ++j) c[j] = v[j];
@@ -517,7 +526,8 @@ template <int DIR, int LO, int HI> __device__ __forceinline__ void fiber_dft(dou
     const int E = fx_exp(key);
     longlong2 x[PG];
 #pragma unroll
-    for (int j = 0; j < PG; ++j) x[j] = mk<longlong2>(fx_in<kFxTop - RHO>(v[j].x, E), fx_in<kFxTop - RHO>(v[j].y, E));
+    for (int j = 0; j < PG; ++j)
+        x[j] = mk<longlong2>(fx_in<kFxTop - 1 - RHO>(v[j].x, E), fx_in<kFxTop - 1 - RHO>(v[j].y, E));
 #pragma unroll
     for (int jh = 0; jh < HI; ++jh) fx_dft<LO, DIR>(x + jh * LO);
     if constexpr (HI > 1) {
@@ -531,7 +541,7 @@ template <int DIR, int LO, int HI> __device__ __forceinline__ void fiber_dft(dou
             for (int jh = 0; jh < HI; ++jh) x[jh * LO + jl] = w[jh];
         }
     }
-    const int e0 = fx_out_exp(E, RHO) + lg_scale;
+    const int e0 = fx_out_exp(E, RHO, 1) + lg_scale;
 #pragma unroll
     for (int j = 0; j < PG; ++j) v[j] = mk<double2>(fx_out(x[j].x, e0), fx_out(x[j].y, e0));
 }

@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(ARITH == kTpF32w ? 512 : 1024) tile_pass_kerne
     for (int64_t t = first; t < end; t += step) {
         __syncthreads();  // tables ready; the previous tile's last stage done with its slots and exponents
         if constexpr (ARITH == kTpFixed) {
-            for (int i = threadIdx.x; i < 1 << a.lg_groups; i += blockDim.x) emax[i] = 0;
+            for (int i = threadIdx.x; i < tp_entries(a); i += blockDim.x) emax[i] = 0;
             __syncthreads();
         }
         const int64_t base = tp_base(a, t);
@@ -97,6 +97,11 @@ cudaError_t launch_t(const TilePass &a, cudaStream_t st) {
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
+    if constexpr (ARITH == kTpFixed) {
+        if (a.shifts)
+            return a.mul ? cudaLaunchKernelEx(&cfg, tile_pass_kernel<ARITH, DIR, kTpMul | kTpShifts>, a)
+                         : cudaLaunchKernelEx(&cfg, tile_pass_kernel<ARITH, DIR, kTpShifts>, a);
+    }
     switch ((a.mul ? kTpMul : 0) | (a.nst == 1 ? kTpSingle : 0)) {
         case 0: return cudaLaunchKernelEx(&cfg, tile_pass_kernel<ARITH, DIR, 0>, a);
         case kTpMul: return cudaLaunchKernelEx(&cfg, tile_pass_kernel<ARITH, DIR, kTpMul>, a);
@@ -120,6 +125,12 @@ cudaError_t prepare_t(TilePass &a) {
                                : prepare_opt<ARITH, DIR, kTpMul>(a, nullptr);
     if (e == cudaSuccess)
         e = a.nst == 1 ? prepare_opt<ARITH, DIR, kTpSingle>(a, &per_sm) : prepare_opt<ARITH, DIR, 0>(a, &per_sm);
+    if constexpr (ARITH == kTpFixed) {
+        if (e == cudaSuccess && a.shifts) {
+            e = prepare_opt<ARITH, DIR, kTpMul | kTpShifts>(a, nullptr);
+            if (e == cudaSuccess) e = prepare_opt<ARITH, DIR, kTpShifts>(a, &per_sm);
+        }
+    }
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
@@ -299,7 +310,6 @@ bool make_tile_pass(int d, const int64_t *n, const int64_t *p, int l0, int l1, i
         TileStage &s = a.st[si];
         s.lg_r = g.bits;
         s.pos = g.pos;
-        s.sh = si + 1 < no ? dg[order[si + 1]].bits : 0;
         s.tw = tw[l];
         s.tw64 = tw64[l];
         for (int b = 0; b < g.bits; ++b) s.rb[b] = slot(1 << (g.pos + b));
@@ -325,10 +335,49 @@ bool make_tile_pass(int d, const int64_t *n, const int64_t *p, int l0, int l1, i
         s.tab = tab;
         if (s.tw_kind) tab += 1 << (g.bits + s.lg_q);
     }
+    if (is_double) {
+        // The shift before each later stage (fixed64.cuh): what any data need, from 2^61.5 after the first stage and from the
+        // others' limit to the stage's own; the largest ones by the groups' sizes, until the
+        // others take kFxFixed bits at most.  A product halves in any case.
+        int need[kTpStages], least[kTpStages], total = 0;
+        auto limit = [&](int si) { return si == 0 || a.st[si].tw_kind ? 61 : 62; };  // and a half
+        for (int si = 1; si < no; ++si) {
+            least[si] = a.st[si - 1].tw_kind ? 1 : 0;
+            need[si] = std::max(least[si], limit(si - 1) + a.st[si].lg_r - limit(si));
+            total += need[si];
+        }
+        if (no > 1 && a.st[no - 1].tw_kind) total += a.st[no - 1].sh = 1;
+        while (total > kFxFixed) {
+            int most = 0;
+            for (int si = 1; si < no; ++si)
+                if (need[si] > least[si] && (!most || need[si] - least[si] > need[most] - least[most])) most = si;
+            if (!most) break;
+            total -= need[most] - least[most];
+            need[most] = least[most];
+            a.st[most].size_in = a.st[most - 1].size_out = ++a.sizes;
+            a.size_lg[a.sizes] = a.st[most].lg_r;
+            a.size_room[a.sizes] = a.st[most].tw_kind ? kFxRoomHalved : kFxRoomNone;
+        }
+        for (int si = 1; si < no; ++si) {
+            (a.st[si - 1].tw_kind ? a.st[si - 1].sh : a.st[si].pre) = need[si];
+            if (a.st[si].pre || a.st[si].size_in) a.shifts = 1;
+        }
+        a.shift = total;
+        for (int si = 0; si < no; ++si) {
+            const TileStage &s = a.st[si];
+            bool one = a.lg_tile - s.lg_r >= 5;
+            for (int b = 0; b < 5; ++b) {
+                const int e = b < s.pos ? b : b + s.lg_r;
+                for (int i = 0; i < a.ngroup; ++i)
+                    if (e >= a.group[i].sh && e < a.group[i].sh + ilog2(a.group[i].mask + 1)) one = false;
+            }
+            a.st[si].warp = one;
+        }
+    }
     const size_t es = is_double ? 16 : 8;
     a.tab_off = no > 1 ? es << a.lg_tile : 0;
     a.emax_off = a.tab_off + tab * es;
-    a.smem = a.emax_off + (is_double ? sizeof(int) << a.lg_groups : 0);
+    a.smem = a.emax_off + (is_double ? sizeof(int) * tp_entries(a) : 0);
     // complex128: one fiber of the first stage per thread (its exponent covers all of them); complex64: 16 values
     a.threads = is_double ? 1 << (a.lg_tile - a.st[0].lg_r) : a.lg_tile > 9 + wide ? 1 << (a.lg_tile - 4 - wide) : 32;
     if (a.once) a.threads = 1 << (a.lg_tile - a.st[0].lg_r);

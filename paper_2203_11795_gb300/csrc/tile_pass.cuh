@@ -39,8 +39,9 @@ namespace fftu {
 // ARITH of a tile pass; kTpF32w: complex64 with radix-32 stages (a kernel of its own, with twice the registers)
 constexpr int kTpF32 = 0, kTpFixed = 1, kTpF64 = 2, kTpF32w = 3;
 // OPT bits: the pointwise product in the last store; twiddles straight from the root tables instead of the stages' shared
-// tables; a pass of one stage; passes that follow one another in one launch (loads from L2).
-constexpr int kTpMul = 1, kTpGlobalTw = 2, kTpSingle = 4, kTpChain = 8;
+// tables; a pass of one stage; passes that follow one another in one launch (loads from L2); complex128 stages that shift
+// their inputs, by their groups' sizes or as any data need (a kernel of its own: the others would lose 2%).
+constexpr int kTpMul = 1, kTpGlobalTw = 2, kTpSingle = 4, kTpChain = 8, kTpShifts = 16;
 template <int ARITH> struct tp_type;
 template <> struct tp_type<kTpF32> { using elem = float2; using work = float2; using tw = float2; };
 template <> struct tp_type<kTpF32w> : tp_type<kTpF32> {};
@@ -133,7 +134,8 @@ __device__ __forceinline__ void tp_twiddles(const TileStageCore &s, int e0, type
 }
 
 // One stage of radix R.  FIRST: from src; LAST: to dst (both: a pass of one digit).  Returns false (kTpFixed, FIRST)
-// when the tile needs FP64 arithmetic.  `key` table: one magnitude key per v (kTpFixed).
+// when the tile needs FP64 arithmetic.  emax (kTpFixed): per group the largest key, then the sizes (fx_size)
+// that some stages leave for the next one.
 template <int ARITH, int DIR, int OPT, int R, bool FIRST, bool LAST, typename P>
 __device__ __forceinline__ bool tp_stage(const P &a, int si, typename tp_type<ARITH>::work *sm,
                                          const typename tp_type<ARITH>::tw *tabs, int *emax,
@@ -142,6 +144,7 @@ __device__ __forceinline__ bool tp_stage(const P &a, int si, typename tp_type<AR
     using T = tp_type<ARITH>;
     using W = typename T::work;
     constexpr int RHO = lg_of<R>();
+    constexpr bool kShifts = ARITH == kTpFixed && (OPT & kTpShifts) != 0;
     int phi0 = threadIdx.x;
     asm volatile("" : "+r"(si), "+r"(phi0));  // per tile: nothing derived from them is kept in registers across tiles
     const auto &s = a.st[si];
@@ -157,6 +160,8 @@ __device__ __forceinline__ bool tp_stage(const P &a, int si, typename tp_type<AR
         int slot = 0;
         if constexpr (!(FIRST && LAST)) slot = tp_slot<ARITH>(a, e0);
         int key = 0;
+        [[maybe_unused]] int *em = nullptr;   // kTpFixed: the group's entries
+        [[maybe_unused]] bool fine = false;  // a fiber of small values in its group (fx_fine)
         if constexpr (FIRST) {
             const unsigned off = a.lg_inner < 0 ? (unsigned)e0
                                                 : (((unsigned)e0 >> a.lg_v) << a.lg_inner) | (e0 & ((1 << a.lg_v) - 1));
@@ -170,27 +175,18 @@ __device__ __forceinline__ bool tp_stage(const P &a, int si, typename tp_type<AR
 #pragma unroll
                     for (int r = 0; r < R; ++r) x[r] = mk<double2>(0.0, 0.0);
                 }
-                unsigned lo = 0;
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int k = fx_key(x[r]);
-                    key = k > key ? k : key;
-                }
-                if (key == 0) {
-#pragma unroll
-                    for (int r = 0; r < R; ++r)
-                        lo |= (unsigned)__double2loint(x[r].x) | (unsigned)__double2loint(x[r].y);
-                }
-                const int bad = !fx_plain(key, lo);
-                int *em = emax + tp_fields(a.group, a.ngroup, (unsigned)e0);
-                if (phi < fibers) atomicMax(em, key);
-                if (__syncthreads_or(bad)) return false;
+                key = fx_keys<R>(x);
+                em = emax + tp_fields(a.group, a.ngroup, (unsigned)e0);
+                if (phi < fibers) fx_raise(em, key, s.warp);
+                if (__syncthreads_or(!fx_plain(key))) return false;
                 if (phi >= fibers) break;
+                const int own = key;
                 key = *em;
-                const int E = fx_exp(key);
+                if constexpr (!LAST) fine = fx_fine(own, key);
+                const int E = fx_exp(key) - (fine ? kFxFine : 0);
 #pragma unroll
                 for (int r = 0; r < R; ++r)
-                    v[r] = mk<longlong2>(fx_in<kFxTop - RHO>(x[r].x, E), fx_in<kFxTop - RHO>(x[r].y, E));
+                    v[r] = mk<longlong2>(fx_in<kFxTop - LAST - RHO>(x[r].x, E), fx_in<kFxTop - LAST - RHO>(x[r].y, E));
             } else {
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[r] = tp_load<OPT>(p + ((size_t)r << a.in_bit));
@@ -200,7 +196,24 @@ __device__ __forceinline__ bool tp_stage(const P &a, int si, typename tp_type<AR
 #pragma unroll
             for (int r = 0; r < R; ++r) v[r] = sm[at(r)];
         }
+        [[maybe_unused]] int sh = 0, shift = FIRST ? 1 : a.shift;  // kTpFixed: of all stages (a first stage alone: one less in K)
+        if constexpr (ARITH == kTpFixed && !FIRST) {
+            if constexpr (LAST || kShifts) em = emax + tp_fields(a.group, a.ngroup, (unsigned)e0);
+            if constexpr (LAST) key = *em;
+            if constexpr (LAST && kShifts) {
+#pragma unroll 1
+                for (int i = 1; i <= a.sizes; ++i) shift += fx_shift(em[i << a.lg_groups], a.size_lg[i], a.size_room[i]);
+            }
+            if constexpr (kShifts) {
+                sh = s.pre;
+                if (s.size_in) sh = fx_shift(em[s.size_in << a.lg_groups], RHO, s.tw_kind ? kFxRoomHalved : kFxRoomNone);
+                if (s.pre || s.size_in) fx_floor<R>(v, sh);
+            }
+        }
         tp_dft<ARITH, DIR, R>(v);
+        if constexpr (kShifts && !FIRST) {
+            if (s.pre || s.size_in) fx_mend<R>(v, sh);
+        }
         if constexpr (LAST) {
             if (s.tw_kind) tp_twiddles<ARITH, DIR, OPT, R>(s, e0, v, tabs);  // phase A: w_n^{k s} of the last axis
             typename T::elem *q;
@@ -208,8 +221,7 @@ __device__ __forceinline__ bool tp_stage(const P &a, int si, typename tp_type<AR
                 if (a.once) __syncthreads();  // every thread has one fiber: all loads of the tile are done
             }
             q = dst + tp_fields(a.out, a.nout, (unsigned)phi);
-            if constexpr (ARITH == kTpFixed && !FIRST) key = emax[tp_fields(a.group, a.ngroup, (unsigned)e0)];
-            [[maybe_unused]] const int x0 = fx_out_exp(fx_exp(key), a.lg_dft) + a.lg_scale;
+            [[maybe_unused]] const int x0 = fx_out_exp(fx_exp(key), a.st[0].lg_r, shift) + a.lg_scale;
             [[maybe_unused]] const auto f = (typename real_of<W>::type)a.scale;
             // kTpMul: the pointwise factor at the same natural index
             [[maybe_unused]] const typename T::elem *m =
@@ -217,24 +229,29 @@ __device__ __forceinline__ bool tp_stage(const P &a, int si, typename tp_type<AR
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 typename T::elem y;
-                if constexpr (ARITH == kTpFixed) {
-                    if (key == 0) v[r] = mk<longlong2>(0, 0);  // no trace of the products' rounding constants
-                    y = mk<double2>(fx_out(v[r].x, x0), fx_out(v[r].y, x0));
-                } else {
-                    y = a.lg_scale != 0 ? cscale(v[r], f) : v[r];
-                }
+                if constexpr (ARITH == kTpFixed) y = mk<double2>(fx_out(v[r].x, x0), fx_out(v[r].y, x0));
+                else y = a.lg_scale != 0 ? cscale(v[r], f) : v[r];
                 if constexpr ((OPT & kTpMul) != 0) y = cmul(y, m[(size_t)r << a.out_bit]);
                 q[(size_t)r << a.out_bit] = y;
             }
         } else {
-            if (s.tw_kind) tp_twiddles<ARITH, DIR, OPT, R>(s, e0, v, tabs);
-            if constexpr (ARITH == kTpFixed) {  // the next stage's scale, where the table did not bring it
-                if ((OPT & kTpGlobalTw) != 0 || s.tw_kind == 0) {
+            if constexpr (ARITH == kTpFixed) {  // the stage's shift for any data, where its table does not bring it
+                if ((OPT & kTpGlobalTw) != 0 && s.tw_kind) {
 #pragma unroll
                     for (int r = 0; r < R; ++r) v[r] = fx_scale_down(v[r], s.sh);
                 } else if (s.tw_kind == 1) {
                     v[0] = fx_scale_down(v[0], s.sh);
                 }
+            }
+            if (s.tw_kind) tp_twiddles<ARITH, DIR, OPT, R>(s, e0, v, tabs);
+            if constexpr (ARITH == kTpFixed && FIRST) {
+                if (fine) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) v[r] = fx_scale_down(v[r], kFxFine);
+                }
+            }
+            if constexpr (kShifts) {
+                if (s.size_out) fx_raise(em + (s.size_out << a.lg_groups), fx_size<R>(v), s.warp);
             }
             TpSlots<std::remove_const_t<std::remove_reference_t<decltype(s)>>, R> at(s, slot);
 #pragma unroll
@@ -276,9 +293,11 @@ __device__ __forceinline__ void tp_tables(const P &a, typename tp_type<ARITH>::t
         const TW *tw = static_cast<const TW *>(s.tw);
         const int n = 1 << (s.lg_r + s.lg_q);
         for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const TW w = tw[tp_exponent(s, (unsigned)i >> s.lg_q, (unsigned)i & ((1u << s.lg_q) - 1))];
-            if constexpr (ARITH == kTpFixed) tabs[s.tab + i] = fx_scale_tw(w, s.sh);
-            else tabs[s.tab + i] = w;
+            TW w = tw[tp_exponent(s, (unsigned)i >> s.lg_q, (unsigned)i & ((1u << s.lg_q) - 1))];
+            if constexpr (ARITH == kTpFixed) {
+                w = fx_scale_tw(w, s.sh);
+            }
+            tabs[s.tab + i] = w;
         }
     }
 }
@@ -301,6 +320,11 @@ __device__ __forceinline__ bool tp_run(const P &a, typename tp_type<ARITH>::work
 template <int DIR, int OPT, typename P>
 __device__ __noinline__ void tp_run_fp64(const P &a, double2 *sm, const double2 *src, double2 *dst) {
     tp_run<kTpF64, DIR, OPT>(a, sm, nullptr, nullptr, src, dst);
+}
+
+// complex128: entries of the exponent groups (tp_stage).
+template <typename P> __host__ __device__ __forceinline__ int tp_entries(const P &a) {
+    return (1 + a.sizes) << a.lg_groups;
 }
 
 // Element offset of tile t.
