@@ -81,7 +81,7 @@ typedef enum {
 } fftu_schedule;
 
 /* Arithmetic of the radix-16 DFT stages of the strided passes (complex64 plans only).
- * NATIVE: FP32 (complex64), or 64-bit fixed point with FP64 where values cannot be scaled (complex128),
+ * NATIVE: FP32 (complex64), or 64-bit fixed point with FP64 around infinities and NaN (complex128),
  * on the CUDA cores.
  * SPLIT_BF16 / SPLIT_FP16: each radix-16 stage of 8 butterflies is a real 32 x 32 contraction on
  * the tensor cores (mma.sync m16n8k16, FP32 accumulation) with both operands split into a 16-bit

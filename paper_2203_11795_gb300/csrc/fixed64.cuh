@@ -33,8 +33,8 @@
 // integer addition to the exponent; done in integer instructions it took 44 of a complex value's 271 in a two-stage
 // pass and the integer pipe was the bound.
 //
-// A group with a component that is infinite, NaN, or too small or large to be scaled (fx_plain) is left to the
-// FP64 path of the caller.
+// A group whose largest component is below 2^-895 or above 2^962 is multiplied by a power of two before its conversion, and its
+// results by the inverse.  One with an infinity or NaN is left to the FP64 path of the caller.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -46,10 +46,11 @@ namespace fftu {
 
 template <> struct real_of<longlong2> { using type = long long; };
 
-// Lowest and highest biased exponent of a group that is scaled: its results stay normal down to
-// 2^-(128 - 63 + 40) of it.
+// Lowest and highest biased exponent of a group that is scaled as it is: its results stay normal down to
+// 2^-(128 - 63 + 40) of it.  Others: multiplied by 2^kFxBoost or 2^-kFxBoost first.
 constexpr int kFxMinExp = 128;
 constexpr int kFxMaxExp = 1984;
+constexpr int kFxBoost = 960;
 // Most bits that shifts for any data may take: 256 points.  Its relative error for one nonzero value is that of FP64 butterflies,
 // 9.4e-17; with 5 bits (512 points) 1.5 times theirs.
 constexpr int kFxFixed = 4;
@@ -71,18 +72,32 @@ template <int R> __device__ __forceinline__ int fx_keys(const double2 *v) {
     }
     return key;
 }
-// Whether values up to this key are served: others need the FP64 path.
+__device__ __forceinline__ bool fx_finite(int key) { return key < 0x7ff00000; }
+// Whether values up to this key are scaled as they are.
 __device__ __forceinline__ bool fx_plain(int key) {
     const int e = key >> 20;
     return key == 0 || (e >= kFxMinExp && e <= kFxMaxExp);
 }
+// The power of two that a group of this key is multiplied by before its conversion (denormals then are ordinary values).
+__device__ __forceinline__ int fx_boost(int key) { return fx_plain(key) ? 0 : (key >> 20) < kFxMinExp ? kFxBoost : -kFxBoost; }
+template <int R> __device__ __forceinline__ void fx_times(double2 *v, int up) {  // v 2^up
+    const double f = __hiloint2double((1023 + up) << 20, 0);
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = mk<double2>(v[r].x * f, v[r].y * f);
+}
+// The key of such a group after the multiplication: the exponent and which it was (bits 31 and 0).
+__device__ __forceinline__ int fx_far_key(int key, int boost) {
+    return (int)(0x80000000u | (unsigned)(max(key >> 20, 1) + boost) << 20 | (boost > 0 ? 1u : 0u));
+}
+__device__ __forceinline__ bool fx_far(int key) { return key < 0; }
+__device__ __forceinline__ int fx_far_boost(int key) { return key & 1 ? kFxBoost : -kFxBoost; }
 // Biased exponent the group is scaled with.
-__device__ __forceinline__ int fx_exp(int key) { return max(key >> 20, kFxMinExp); }
+__device__ __forceinline__ int fx_exp(int key) { return max((key >> 20) & 0x7ff, kFxMinExp); }
 
 // Whether a fiber of the first stage whose own values have this key holds them at 2^kFxFine times its group's scale, up to its store:
 // all of them are that much smaller than the largest of the group (a point source elsewhere), which would cost them their low bits.
 constexpr int kFxFine = 3;
-__device__ __forceinline__ bool fx_fine(int own, int group) { return (own >> 20) + kFxFine <= fx_exp(group); }
+__device__ __forceinline__ bool fx_fine(int own, int group) { return (own >> 20) + kFxFine <= fx_exp(group) && !fx_far(group); }
 
 constexpr int kFxTop = 60;  // K + rho of a first stage that others follow
 
@@ -92,7 +107,7 @@ template <int K> __device__ __forceinline__ long long fx_in(double x, int E) {
     const int hi = __double2hiint(x);
     const unsigned lo = (unsigned)__double2loint(x);
     const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
-    const int d = E - ((hi >> 20) & 0x7ff);  // >= 0; denormals: d >= kFxMinExp, shifted out
+    const int d = E - ((hi >> 20) & 0x7ff);  // >= 0; denormals of groups not boosted: d >= kFxMinExp, shifted out
     const long long m = (long long)(((((unsigned long long)mh << 32) | lo) << (K - 52)) >> min(d, 63));
     return hi < 0 ? -m : m;
 }

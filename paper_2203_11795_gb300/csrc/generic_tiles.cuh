@@ -384,7 +384,14 @@ __device__ __forceinline__ bool fx_stage(longlong2 *sm, const int4 *__restrict__
         }
     }
     if constexpr (FIRST) {
-        if (__syncthreads_or(bad)) return false;
+        if (__syncthreads_or(bad)) {  // rare: some values, though perhaps no column, are out of range
+            int beyond = 0;
+            for (int c = tid; c < cols; c += nthreads) beyond |= !fx_finite(emax[c]);
+            if (__syncthreads_or(beyond)) return false;
+            for (int c = tid; c < cols; c += nthreads)
+                if (const int up = fx_boost(emax[c])) emax[c] = fx_far_key(emax[c], up);
+            __syncthreads();
+        }
     } else {
         __syncthreads();
     }
@@ -402,6 +409,7 @@ __device__ __forceinline__ bool fx_stage(longlong2 *sm, const int4 *__restrict__
                 double2 x[R];
 #pragma unroll
                 for (int r = 0; r < R; ++r) x[r] = fx_bits(v[q][r]);
+                if (fx_far(key)) fx_times<R>(x, fx_far_boost(key));
 #pragma unroll
                 for (int r = 0; r < R; ++r)
                     v[q][r] = mk<longlong2>(fx_in<kFxTop - RHO>(x[r].x, E), fx_in<kFxTop - RHO>(x[r].y, E));
@@ -453,14 +461,16 @@ __device__ __forceinline__ void axis_tile_fx(const AxisPass &a, int64_t t, doubl
     for (int Ns = kFirst, si = 1; Ns < a.len; Ns *= 8, ++si) fx_stage<DIR, 8, false>(fx, tw, a, Ns, si, emax, tid, nt);
     // the columns' exponents; 1/N is a power of two and goes into them
     const int lg_scale = (__double2hiint(a.scale) >> 20) - 1023;
+    int far = 0;
     for (int c = tid; c < cols; c += nt) {
         const int key = emax[c];
+        far |= fx_far(key);
         int shift = 1;
         for (int i = 1; i < a.nstages; ++i) shift += fx_shift(emax[i * cols + c], 3, kFxRoomProduct);
         const int e0 = fx_out_exp(fx_exp(key), lg_of<kFirst>(), shift) + lg_scale;
-        emax[c] = e0;
+        emax[c] = e0 * 4 + (!fx_far(key) ? 0 : fx_far_boost(key) > 0 ? 1 : 2);
     }
-    __syncthreads();
+    far = __syncthreads_or(far);
     for (int e = tid; e < a.tile; e += nt) {
         int lpo, v;
         if (a.contiguous) {
@@ -487,9 +497,13 @@ __device__ __forceinline__ void axis_tile_fx(const AxisPass &a, int64_t t, doubl
             gp = o.c0 + cl + ((int64_t)(lpo >> a.lg_Gt) << a.lg_G);
         }
         const int col = a.contiguous ? (v << a.lg_Gt) + cl : (cl << a.lg_V) + v;
-        const int e0 = emax[col];
+        const int e0 = emax[col] >> 2;
         const int64_t g = a.contiguous ? o.gbase + (int64_t)v * a.nl + gp : o.gbase + gp * a.inner + v;
         dst[g] = mk<double2>(fx_out(x.x, e0), fx_out(x.y, e0));
+        if (far) {  // some column was multiplied
+            const int up = emax[col] & 3;
+            if (up) fx_times<1>(dst + g, up == 1 ? -kFxBoost : kFxBoost);
+        }
     }
     __syncthreads();
 }

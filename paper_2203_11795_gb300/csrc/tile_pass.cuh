@@ -178,7 +178,15 @@ __device__ __forceinline__ bool tp_stage(const P &a, int si, typename tp_type<AR
                 key = fx_keys<R>(x);
                 em = emax + tp_fields(a.group, a.ngroup, (unsigned)e0);
                 if (phi < fibers) fx_raise(em, key, s.warp);
-                if (__syncthreads_or(!fx_plain(key))) return false;
+                if (__syncthreads_or(!fx_plain(key))) {  // rare: a fiber, though perhaps no group, is out of range
+                    const int group = phi < fibers ? *em : 0, up = fx_boost(group);
+                    if (__syncthreads_or(!fx_finite(group))) return false;
+                    if (up) {
+                        fx_times<R>(x, up);
+                        *em = key = fx_far_key(group, up);
+                    }
+                    __syncthreads();
+                }
                 if (phi >= fibers) break;
                 const int own = key;
                 key = *em;
@@ -223,6 +231,7 @@ __device__ __forceinline__ bool tp_stage(const P &a, int si, typename tp_type<AR
             q = dst + tp_fields(a.out, a.nout, (unsigned)phi);
             [[maybe_unused]] const int x0 = fx_out_exp(fx_exp(key), a.st[0].lg_r, shift) + a.lg_scale;
             [[maybe_unused]] const auto f = (typename real_of<W>::type)a.scale;
+            [[maybe_unused]] const bool far = ARITH == kTpFixed && fx_far(key);
             // kTpMul: the pointwise factor at the same natural index
             [[maybe_unused]] const typename T::elem *m =
                 (OPT & kTpMul) ? static_cast<const typename T::elem *>(a.mul) + (q - static_cast<typename T::elem *>(a.dst)) : nullptr;
@@ -231,8 +240,20 @@ __device__ __forceinline__ bool tp_stage(const P &a, int si, typename tp_type<AR
                 typename T::elem y;
                 if constexpr (ARITH == kTpFixed) y = mk<double2>(fx_out(v[r].x, x0), fx_out(v[r].y, x0));
                 else y = a.lg_scale != 0 ? cscale(v[r], f) : v[r];
-                if constexpr ((OPT & kTpMul) != 0) y = cmul(y, m[(size_t)r << a.out_bit]);
+                if constexpr ((OPT & kTpMul) != 0) {
+                    if (!far) y = cmul(y, m[(size_t)r << a.out_bit]);
+                }
                 q[(size_t)r << a.out_bit] = y;
+            }
+            if constexpr (ARITH == kTpFixed) {
+                if (far) {  // rare: the stored values are read again, which leaves the loop above as it is without
+#pragma unroll 1
+                    for (int r = 0; r < R; ++r) {
+                        double2 *y = q + ((size_t)r << a.out_bit);
+                        fx_times<1>(y, -fx_far_boost(key));
+                        if constexpr ((OPT & kTpMul) != 0) *y = cmul(*y, m[(size_t)r << a.out_bit]);
+                    }
+                }
             }
         } else {
             if constexpr (ARITH == kTpFixed) {  // the stage's shift for any data, where its table does not bring it
