@@ -594,7 +594,7 @@ def run_ours(args):
             "roofline": roofline,
             "cpu_baseline": cpu,
             "e2e": e2e,
-            "gpu_launches": args.steps * 2 * (la + lb),
+            "gpu_launches": args.steps * 2 * fftu.fftu_exec_launches(fwd.handle),
             "clocks": clocks,
             "round_trip_rel_l2": rt_err,
             "forward_vs_fp32_stages_rel_l2": vs_native,
@@ -879,7 +879,7 @@ def run_pointwise(args):
             "roofline": {"bound": "hbm", "achieved": value / world, "peak": peak, "unit": "GB/s",
                          "frac": value / world / peak, "traffic": None, "kernel": "whole step",
                          "peak_source": f"{peak_kind} hbm_gbs"},
-            "gpu_launches": args.steps * 2 * (fwd.info["launches_phase_a"] + fwd.info["launches_phase_b"]),
+            "gpu_launches": args.steps * 2 * fftu.fftu_exec_launches(fwd.handle),
             "clocks": clocks,
         }
     fail = None if err < 1e-5 else f"fused and separate convolutions differ ({err:.3g})"
@@ -969,7 +969,7 @@ def run_batch(args):
     fftu.fftu_batch_check_status(bi)
     rt = max(float((torch.linalg.vector_norm(z - x) / torch.linalg.vector_norm(x)).item()) for x, z in zip(xs, zs))
     ms_loop = timed(per_plan_step, max(1, args.steps // 4))
-    launches_loop = sum(q.info["launches_phase_a"] + q.info["launches_phase_b"] for q in fwd + inv)
+    launches_loop = sum(fftu.fftu_exec_launches(q.handle) for q in fwd + inv)
 
     e2e = None
     if not args.no_e2e:

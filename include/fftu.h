@@ -127,8 +127,8 @@ typedef struct {
     int dtype;                 /* fftu_dtype */
     int dir;                   /* fftu_dir */
     int schedule;              /* schedule in use (fftu_schedule, never AUTO) */
-    int launches_phase_a;      /* kernel launches one phase A takes */
-    int launches_phase_b;      /* kernel launches one phase B takes */
+    int launches_phase_a;      /* kernel launches of FFTU_PHASE_A alone (a whole transform: fftu_exec_launches) */
+    int launches_phase_b;      /* kernel launches of FFTU_PHASE_B alone */
     int64_t N;                 /* number of elements */
     int64_t alg_bytes;         /* algorithmic HBM bytes per transform: 4 * N * sizeof(element) */
     int64_t table_bytes;       /* device bytes of twiddle tables owned by the plan */
@@ -224,6 +224,10 @@ fftu_status fftu_destroy(fftu_handle plan);
 
 /* Describe a plan (sizes, schedule, launches, byte counts). */
 fftu_status fftu_plan_info(fftu_handle plan, fftu_info *info);
+
+/* Kernel launches of one fftu_exec (out of place).  On a grid that the library chose this can be less than
+ * launches_phase_a + launches_phase_b, which are those of fftu_exec_phase: see fftu_exec_phase. */
+fftu_status fftu_exec_launches(fftu_handle plan, int *launches);
 
 /* Read and clear the plan's device status word (bounded waits and device
  * checks write it).  Synchronises with the plan's last use.  Returns FFTU_OK,

@@ -31,7 +31,7 @@ STATUS_NAMES = {0: "FFTU_OK", 1: "FFTU_ERR_ARG", 2: "FFTU_ERR_DIVISIBILITY", 3: 
 
 # Every entry point the header declares (checked by the test suite).
 EXPORTS = ("fftu_plan", "fftu_plan_ex", "fftu_exec", "fftu_exec_phase", "fftu_exec_pointwise", "fftu_destroy",
-           "fftu_plan_info",
+           "fftu_plan_info", "fftu_exec_launches",
            "fftu_check_device_status", "fftu_exec_noalloc", "fftu_noalloc_check_status",
            "fftu_noalloc_selftest_timeout", "fftu_batch_create", "fftu_batch_exec",
            "fftu_batch_check_status", "fftu_batch_destroy", "fftu_wisdom_export", "fftu_wisdom_import",
@@ -108,6 +108,7 @@ def _load_library() -> ctypes.CDLL:
     lib.fftu_exec_pointwise.argtypes = [h, h, vp, vp, vp, vp, vp]
     lib.fftu_destroy.argtypes = [h]
     lib.fftu_plan_info.argtypes = [h, ctypes.POINTER(fftu_info)]
+    lib.fftu_exec_launches.argtypes = [h, ctypes.POINTER(ctypes.c_int)]
     lib.fftu_check_device_status.argtypes = [h]
     lib.fftu_exec_noalloc.argtypes = [ctypes.c_int, i64p, i64p, ctypes.c_int, ctypes.c_int, vp, vp, vp]
     lib.fftu_noalloc_check_status.argtypes = [vp]
@@ -135,7 +136,7 @@ def _load_library() -> ctypes.CDLL:
     lib.fftu_last_error.restype = ctypes.c_char_p
     lib.fftu_version.restype = ctypes.c_char_p
     for name in ("fftu_plan", "fftu_plan_ex", "fftu_exec", "fftu_exec_phase", "fftu_exec_pointwise", "fftu_destroy",
-                 "fftu_plan_info", "fftu_check_device_status", "fftu_exec_noalloc", "fftu_noalloc_check_status",
+                 "fftu_plan_info", "fftu_exec_launches", "fftu_check_device_status", "fftu_exec_noalloc", "fftu_noalloc_check_status",
                  "fftu_noalloc_selftest_timeout", "fftu_batch_create",
                  "fftu_batch_exec", "fftu_batch_check_status", "fftu_batch_destroy", "fftu_wisdom_export",
                  "fftu_wisdom_import", "fftu_wisdom_forget", "fftu_workspace_size", "fftu_set_workspace",
@@ -220,6 +221,13 @@ def fftu_plan_info(plan: int) -> dict:
             "table_bytes": info.table_bytes, "workspace_bytes": info.workspace_bytes, "tuned": info.tuned,
             "precision": info.precision, "workspace_need": info.workspace_need, "layout": info.layout,
             "workspace_mode": info.workspace_mode, "tile": info.tile, "radix": info.radix}
+
+
+def fftu_exec_launches(plan: int) -> int:
+    """Kernel launches of one fftu_exec (out of place)."""
+    k = ctypes.c_int()
+    _check(_lib.fftu_exec_launches(plan, ctypes.byref(k)), "fftu_exec_launches")
+    return k.value
 
 
 def fftu_check_device_status(plan: int) -> None:

@@ -1405,6 +1405,18 @@ fftu_status fftu_plan_info(fftu_handle h, fftu_info *info) {
     return FFTU_OK;
 }
 
+fftu_status fftu_exec_launches(fftu_handle h, int *launches) {
+    using namespace fftu;
+    if (!h || !h->impl || !launches) {
+        set_err("plan and launches must be non-NULL");
+        return FFTU_ERR_ARG;
+    }
+    const Plan *pl = h->impl;
+    *launches = pl->whole.empty() ? kernel_count(pl->phase_a) + kernel_count(pl->phase_b) : (int)pl->whole.size();
+    if (pl->layout == FFTU_LAYOUT_CYCLIC) *launches += 2;  // the permutations
+    return FFTU_OK;
+}
+
 fftu_status fftu_workspace_size(fftu_handle h, size_t *bytes) {
     using namespace fftu;
     if (!h || !h->impl || !bytes) {

@@ -200,9 +200,8 @@ size_t plan_device_bytes(fftu_handle h) {
 }
 
 int plan_launches(fftu_handle h) {
-    fftu_info info;
-    if (fftu_plan_info(h, &info) != FFTU_OK) return 0;
-    return info.launches_phase_a + info.launches_phase_b;
+    int launches = 0;
+    return fftu_exec_launches(h, &launches) == FFTU_OK ? launches : 0;
 }
 
 void note_cuda_error(fftu_server_st *S, cudaError_t e, int site) {
