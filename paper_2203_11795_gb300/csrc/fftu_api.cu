@@ -455,12 +455,6 @@ bool choose_tile_pass(int d, const int64_t *n, const int64_t *p, int l1, int l_m
     const int max_g = contiguous ? target : max_tile - need_v;  // several axes
     if (lg_g + need_v > max_tile || (contiguous && lg_g > 12)) return false;
     while (l0 > l_min && l1 - l0 < 2 && lg_g + ilog2(n[l0 - 1]) <= max_g) lg_g += ilog2(n[--l0]);
-    // complex128: two contiguous axes of 64 points in a tile of 4096 elements where such tiles fill the GPU: the axes share
-    // the conversions to and from fixed point, a sixth of a pass' instructions (64^4 635 -> 601 us).  No gain for other
-    // lengths, whose digits are uneven or reach the long axis anyway (256 x 16 x 16 x 256 697 -> 724 us, 64 x 64 x 8 x 512
-    // 590 -> 720).
-    if (is_double && contiguous && !batched && l0 == l1 && l0 > l_min && lg_g == 6 && n[l0 - 1] == 64 && (N >> 12) >= 304)
-        --l0;
     for (;; ++l0) {  // fewer axes when the stages do not work out
         while (l0 < l1 && n[l0] == 1) ++l0;
         int64_t outer = 1;
