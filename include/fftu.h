@@ -116,7 +116,10 @@ typedef struct {
                             long line that fit), a power of two in [1024, 8192] (complex128: [1024, 4096]);
                             0 = default (4096 / 2048) */
     int radix;           /* strided passes' stages: 8 = radix 8 after one smaller first stage (default,
-                            also 0); 16 = radix-16 stages then one stage of the remaining factor */
+                            also 0); 16 = radix-16 stages then one stage of the remaining factor.
+                            tile and radix choose among forms of the strided passes (schedules GENERIC and
+                            GENERIC_A, split precision) and have no effect on the fused, register-resident
+                            and tile passes that AUTO and FUSED take instead where they apply */
     int reserved[1];     /* must be zero */
 } fftu_options;
 
@@ -138,8 +141,8 @@ typedef struct {
     int64_t workspace_need;    /* device bytes of workspace the plan uses (owned or supplied) */
     int layout;                /* fftu_layout */
     int workspace_mode;        /* fftu_workspace_mode */
-    int tile;                  /* whole-line tile target of the strided passes (elements) */
-    int radix;                 /* 8 or 16: the strided passes' stage radix */
+    int tile;                  /* whole-line tile target of the strided passes (elements), if the plan runs any */
+    int radix;                 /* 8 or 16: the strided passes' stage radix, if the plan runs any */
 } fftu_info;
 
 /*
@@ -198,6 +201,9 @@ fftu_status fftu_exec(fftu_handle plan, const void *in, void *out, void *stream)
  *                 their p_1 x ... x p_d DFT (Superstep 2), scaled by 1/N for
  *                 the inverse.
  *   FFTU_PHASE_ALL: same as fftu_exec.
+ * On a grid of the caller's the two phases one after the other give the bits of fftu_exec.  On one that
+ * the library chose (p == NULL, schedule AUTO, native precision) fftu_exec may take other passes, over
+ * whole axes: the same transform, rounded in another order.
  */
 fftu_status fftu_exec_phase(fftu_handle plan, fftu_phase phase, const void *in, void *out,
                             void *stream);
@@ -212,8 +218,9 @@ fftu_status fftu_exec_phase(fftu_handle plan, fftu_phase phase, const void *in, 
  *   mul       device array of N elements, the multiplier in the frequency domain, natural order.
  *   tmp       device array of N elements for the spectrum; may equal in; must differ from out and mul.
  *   out       device array of N elements; may equal in.
- * When the forward plan's phase B is the fused 3D kernel, the product happens in its store (one extra
- * read of mul, no extra pass); otherwise one elementwise pass follows phase B.  Stream-ordered.
+ * Where the forward plan runs whole-axis passes (see fftu_exec_phase), or its phase B is the fused 3D
+ * kernel or complex128, the product happens in the last store (one extra read of mul, no extra pass);
+ * otherwise one elementwise pass follows.  Stream-ordered.
  */
 fftu_status fftu_exec_pointwise(fftu_handle fwd, fftu_handle inv, const void *in, const void *mul, void *tmp,
                                 void *out, void *stream);
@@ -281,12 +288,13 @@ fftu_status fftu_noalloc_selftest_timeout(double limit_s, void *stream);
 /*
  * Batches: many transforms of different shapes in one persistent kernel launch.
  * fftu_batch_create -- build a batch from `count` (1..128) existing plans with the same dtype,
- *   direction and device.  Every pass of every plan becomes a job (phase A's strided sub-FFT passes,
- *   then phase B, Algorithm 2.3); a persistent kernel takes their tiles in pass-major order and a tile
- *   of pass k waits (bounded) for pass k - 1 of the same transform.  Plans whose phase A alternates with
+ *   direction and device.  Every pass of every plan becomes a job (where all of them are plans of
+ *   whole-axis passes those, else phase A's strided sub-FFT passes, then phase B, Algorithm 2.3); a
+ *   persistent kernel takes their tiles in pass-major order and a tile of pass k waits (bounded) for
+ *   pass k - 1 of the same transform.  Plans whose phase A alternates with
  *   a workspace (a line longer than a tile) are not batched (FFTU_ERR_UNSUPPORTED).  The batch reads the
- *   plans' twiddle tables: destroy the batch before its plans.  It owns a small device job table and
- *   counters.
+ *   plans' twiddle tables: destroy the batch before its plans.  It owns a device job table, counters and, for
+ *   whole-axis passes, up to 8 KB of twiddles a job.
  * fftu_batch_exec -- run the batch on `stream`: ins[i] -> outs[i] (device arrays of plan i's size,
  *   16-byte aligned; outs[i] may equal ins[i]; arrays of different transforms must not overlap).  No host
  *   synchronisation: the counters are cleared on the stream, so the call can be captured into a CUDA graph.

@@ -174,7 +174,8 @@ struct TileParams {
 
 constexpr int kTileBatchThreads = 256;
 // The jobs' tables are copied to shared memory with their descriptors up to this size (four CTAs of 32 KB tiles per SM);
-// with a longer table in the batch (axes of 512 points and more) its passes read the roots instead.
+// with a longer table anywhere in the batch (complex64 axes from 1024 points, complex128 ones from 512) all of its passes
+// read the roots instead.
 constexpr int kTileBatchTable = 512;  // 16-byte units
 
 template <int ARITH>

@@ -637,9 +637,9 @@ fftu_status build_whole(Plan &pl) {
         cudaError_t e = prepare_tile_pass(a, pl.dtype == FFTU_C128, pl.dir);
         if (e != cudaSuccess) return cuda_fail(e, "tile pass attributes");
     }
-    // complex64: between radix-32 passes, which hold all registers of an SM with half the threads, a CTA per tile is the
-    // slower form of the others (64 x 2048 x 512: 705 us against 645 persistent, 64 x 512 x 512 162 and 157; without
-    // radix-32 passes 64^4 163 and 195, 64 x 64 x 4096 172 and 198)
+    // complex64: beside radix-32 passes a CTA per tile measured slower for the others (64 x 2048 x 512: 705 us against 645
+    // persistent, 64 x 512 x 512 162 and 157), without them faster (64^4 163 and 195, 64 x 64 x 4096 172 and 198); why was not
+    // found out
     bool wide = false;
     for (const TilePass &a : steps) wide = wide || a.wide;
     for (TilePass &a : steps)
