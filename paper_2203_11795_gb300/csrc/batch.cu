@@ -154,6 +154,7 @@ static_assert(offsetof(TileTask, st) == offsetof(TilePass, st));
 void fill_task(const TilePass &p, TileTask &t) {
     std::memcpy(static_cast<void *>(&t), &p, offsetof(TilePass, st));
     for (int i = 0; i < kTpStages; ++i) t.st[i] = p.st[i];
+    t.shifts = p.shifts;
 }
 
 struct TileParams {

@@ -129,7 +129,10 @@ struct PhaseBFused {
 // Tile pass (see tile_pass.cuh): every position of axes l0 .. l1 for 2^lg_v adjacent inner (or, on contiguous memory,
 // outer) positions per tile.  Whole axes (the full F_{n_l}), or phase A on them (F_{n_l/p_l} on every class, twiddle,
 // Put).  May be in place.
-constexpr int kTpStages = 8, kTpFields = 8;
+// At most 6 stages: 14 bits of up to three axes in digits of 3 bits and more but for each axis' last.  A pass is a kernel's
+// parameter, and the order of its fields shows in small arrays: 1024 x 1024 complex64 takes 18.2 us with this one, 18.5 to 19.8
+// with the fields of complex128 between the others or the stage's fields in another order.
+constexpr int kTpStages = 6, kTpFields = 8;
 struct BitField {
     int sh, mask, dst;  // ((x >> sh) & mask) << dst
 };
@@ -140,20 +143,28 @@ struct TileStageCore {
     int lo, lg_q;       // twiddle column q in [2^lg_q]: kind 1 j = tile bits [lo, lo + lg_q); kind 2 class s = tile bits
                         // [lo, lo + lg_p) and the axis' bits above the digit
     int lg_p, lg_step;  // kind 1: exponent r j 2^lg_step; kind 2: exponent (k_prev + r 2^lg_step) s
+    int sh;             // complex128 (fixed64.cuh): shift of the stage's results for any data, through its twiddles
     int nk;             // kind 2: k_prev = fields k[] of the bits above the digit
     BitField k[2];
     int tab;            // the table's place in shared memory (elements): entry (r, q) at tab + (r << lg_q) + q
     const void *tw;     // w_n^e (complex128: in fixed point)
     const void *tw64;   // complex128: w_n^e as double2
-    // complex128 (fixed64.cuh)
-    int sh, pre;        // shifts for any data: of the stage's results, through its twiddles, and of its inputs
-    int size_in;        // shift of its inputs by the groups' sizes in entries size_in (0: none)
-    int size_out;       // where it leaves its results' sizes for the next stage
-    int warp;           // the fibers of a warp are of one exponent group
     int rb[5];          // shared slot of 1 << (pos + b)
+    // complex128
+    int8_t pre;         // shift of the stage's inputs for any data
+    int8_t size_in;     // shift of its inputs by the groups' sizes in entries size_in (0: none)
+    int8_t size_out;    // where it leaves its results' sizes for the next stage
+    int8_t warp;        // the fibers of a warp are of one exponent group
 };
 struct TileStage : TileStageCore {
     int rx[32];         // shared slot of r << pos
+};
+// complex128: how the stages of a pass shift their inputs.
+struct TileShifts {
+    int any;            // whether one does (pre, size_in)
+    int sizes;          // stages that do it by their groups' sizes: entries 1 .. sizes,
+    int lg[kTpStages], room[kTpStages];  // log2 of the stage's points, room that it leaves
+    int fixed;          // sum of the stages' sh and pre
 };
 template <typename STAGE> struct TilePassOf {
     const void *src;
@@ -173,14 +184,11 @@ template <typename STAGE> struct TilePassOf {
     BitField last[kTpFields], out[kTpFields];  // last stage: thread index -> tile index, -> element offset
     BitField group[kTpFields];                 // complex128: tile index -> exponent group (one per sub-DFT)
     int lg_groups;
-    int shifts;                                // complex128: some stage shifts its inputs (pre, size_in)
-    int sizes;                                 // stages that do it by their groups' sizes: entries 1 .. sizes,
-    int size_lg[kTpStages], size_room[kTpStages];  // log2 of the stage's points, room that it leaves
-    int shift;                                 // sum of the stages' sh and pre
     int lg_scale;
     double scale;       // 2^lg_scale
     size_t tab_off, emax_off, smem;
     STAGE st[kTpStages];
+    TileShifts shifts;
 };
 using TilePass = TilePassOf<TileStage>;      // of a launch of one pass
 using TileTask = TilePassOf<TileStageCore>;  // of a batch, whose descriptors are copied to shared memory for each tile

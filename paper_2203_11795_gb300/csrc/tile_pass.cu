@@ -98,7 +98,7 @@ cudaError_t launch_t(const TilePass &a, cudaStream_t st) {
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     if constexpr (ARITH == kTpFixed) {
-        if (a.shifts)
+        if (a.shifts.any)
             return a.mul ? cudaLaunchKernelEx(&cfg, tile_pass_kernel<ARITH, DIR, kTpMul | kTpShifts>, a)
                          : cudaLaunchKernelEx(&cfg, tile_pass_kernel<ARITH, DIR, kTpShifts>, a);
     }
@@ -126,7 +126,7 @@ cudaError_t prepare_t(TilePass &a) {
     if (e == cudaSuccess)
         e = a.nst == 1 ? prepare_opt<ARITH, DIR, kTpSingle>(a, &per_sm) : prepare_opt<ARITH, DIR, 0>(a, &per_sm);
     if constexpr (ARITH == kTpFixed) {
-        if (e == cudaSuccess && a.shifts) {
+        if (e == cudaSuccess && a.shifts.any) {
             e = prepare_opt<ARITH, DIR, kTpMul | kTpShifts>(a, nullptr);
             if (e == cudaSuccess) e = prepare_opt<ARITH, DIR, kTpShifts>(a, &per_sm);
         }
@@ -336,33 +336,38 @@ bool make_tile_pass(int d, const int64_t *n, const int64_t *p, int l0, int l1, i
         if (s.tw_kind) tab += 1 << (g.bits + s.lg_q);
     }
     if (is_double) {
-        // The shift before each later stage (fixed64.cuh): what any data need, from 2^61.5 after the first stage and from the
-        // others' limit to the stage's own; the largest ones by the groups' sizes, until the
-        // others take kFxFixed bits at most.  A product halves in any case.
+        // The shift before each later stage (fixed64.cuh): what any data need, from 2^61.5 after the first stage, to stay within
+        // the stages' limits; the largest ones by the groups' sizes, until the others take kFxFixed bits at most.  A product
+        // halves in any case.
         int need[kTpStages], least[kTpStages], total = 0;
-        auto limit = [&](int si) { return si == 0 || a.st[si].tw_kind ? 61 : 62; };  // and a half
-        for (int si = 1; si < no; ++si) {
-            least[si] = a.st[si - 1].tw_kind ? 1 : 0;
-            need[si] = std::max(least[si], limit(si - 1) + a.st[si].lg_r - limit(si));
-            total += need[si];
-        }
-        if (no > 1 && a.st[no - 1].tw_kind) total += a.st[no - 1].sh = 1;
-        while (total > kFxFixed) {
-            int most = 0;
-            for (int si = 1; si < no; ++si)
+        bool sized[kTpStages] = {};
+        for (;;) {
+            int bound = 61, most = 0;  // and a half
+            total = no > 1 && a.st[no - 1].tw_kind ? 1 : 0;
+            for (int si = 1; si < no; ++si) {
+                const int limit = a.st[si].tw_kind ? 61 : 62, grown = bound + a.st[si].lg_r;
+                least[si] = a.st[si - 1].tw_kind ? 1 : 0;
+                need[si] = sized[si] ? least[si] : std::max(least[si], grown - limit);
+                bound = std::min(grown - need[si], limit);
+                total += need[si];
                 if (need[si] > least[si] && (!most || need[si] - least[si] > need[most] - least[most])) most = si;
-            if (!most) break;
-            total -= need[most] - least[most];
-            need[most] = least[most];
-            a.st[most].size_in = a.st[most - 1].size_out = ++a.sizes;
-            a.size_lg[a.sizes] = a.st[most].lg_r;
-            a.size_room[a.sizes] = a.st[most].tw_kind ? kFxRoomHalved : kFxRoomNone;
+            }
+            if (total <= kFxFixed || !most) break;
+            sized[most] = true;
         }
+        if (no > 1 && a.st[no - 1].tw_kind) a.st[no - 1].sh = 1;
+        for (int si = 1; si < no; ++si)
+            if (sized[si]) {
+                a.st[si].size_in = a.st[si - 1].size_out = (int8_t)++a.shifts.sizes;
+                a.shifts.lg[a.shifts.sizes] = a.st[si].lg_r;
+                a.shifts.room[a.shifts.sizes] = a.st[si].tw_kind ? kFxRoomHalved : kFxRoomNone;
+            }
         for (int si = 1; si < no; ++si) {
-            (a.st[si - 1].tw_kind ? a.st[si - 1].sh : a.st[si].pre) = need[si];
-            if (a.st[si].pre || a.st[si].size_in) a.shifts = 1;
+            if (a.st[si - 1].tw_kind) a.st[si - 1].sh = need[si];
+            else a.st[si].pre = (int8_t)need[si];
+            if (a.st[si].pre || a.st[si].size_in) a.shifts.any = 1;
         }
-        a.shift = total;
+        a.shifts.fixed = total;
         for (int si = 0; si < no; ++si) {
             const TileStage &s = a.st[si];
             bool one = a.lg_tile - s.lg_r >= 5;

@@ -204,13 +204,14 @@ __device__ __forceinline__ bool tp_stage(const P &a, int si, typename tp_type<AR
 #pragma unroll
             for (int r = 0; r < R; ++r) v[r] = sm[at(r)];
         }
-        [[maybe_unused]] int sh = 0, shift = FIRST ? 1 : a.shift;  // kTpFixed: of all stages (a first stage alone: one less in K)
+        [[maybe_unused]] int sh = 0, shift = FIRST ? 1 : a.shifts.fixed;  // kTpFixed: of all stages (a first stage alone: one less in K)
         if constexpr (ARITH == kTpFixed && !FIRST) {
             if constexpr (LAST || kShifts) em = emax + tp_fields(a.group, a.ngroup, (unsigned)e0);
             if constexpr (LAST) key = *em;
             if constexpr (LAST && kShifts) {
 #pragma unroll 1
-                for (int i = 1; i <= a.sizes; ++i) shift += fx_shift(em[i << a.lg_groups], a.size_lg[i], a.size_room[i]);
+                for (int i = 1; i <= a.shifts.sizes; ++i)
+                    shift += fx_shift(em[i << a.lg_groups], a.shifts.lg[i], a.shifts.room[i]);
             }
             if constexpr (kShifts) {
                 sh = s.pre;
@@ -345,7 +346,7 @@ __device__ __noinline__ void tp_run_fp64(const P &a, double2 *sm, const double2 
 
 // complex128: entries of the exponent groups (tp_stage).
 template <typename P> __host__ __device__ __forceinline__ int tp_entries(const P &a) {
-    return (1 + a.sizes) << a.lg_groups;
+    return (1 + a.shifts.sizes) << a.lg_groups;
 }
 
 // Element offset of tile t.
