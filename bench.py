@@ -1021,7 +1021,7 @@ def run_batch(args):
                        "l2": "arrays total more than L2 but part of a step's working set stays L2-resident",
                        "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                         "frac": achieved / peak, "traffic": None, "kernel": "batch_kernel",
+                         "frac": achieved / peak, "traffic": None, "kernel": "tile_batch_kernel",
                          "peak_source": f"{peak_kind} hbm_gbs"},
             "per_plan_loop": {"ms_per_step": ms_loop, "gpu_launches_per_step": launches_loop,
                               "value": whole_job_value(step_bytes, ms_loop, world)},
@@ -1092,6 +1092,38 @@ def run_secondary(args):
     return out
 
 
+# What the printed line keeps of the long parts of a record; the rest goes to stderr.  A reader of the line's end (or of a
+# few thousand characters of it) still gets the whole line.
+SHORT = {
+    "plan": ("schedule", "precision", "tuned"),
+    "roofline": ("bound", "achieved", "peak", "unit", "frac", "kernel", "peak_source", "step_frac", "phase_ms"),
+    "cpu_baseline": ("value", "unit", "cores", "kind", "seconds_per_rep"),
+    "cufft_context": ("ms_per_step", "value", "unit"),
+    "serving": ("requests", "offered_rate_per_s", "achieved_rate_per_s", "p50_ms", "p99_ms", "gbs_algorithmic", "failed", "error"),
+}
+
+
+def headline(line):
+    """The record with its long parts reduced to their figures."""
+    out = {}
+    for k, v in line.items():
+        if k in SHORT and isinstance(v, dict):
+            out[k] = {x: v[x] for x in SHORT[k] if x in v}
+        elif k == "secondary":
+            out[k] = {name: {x: e[x] for x in ("value", "ms_per_step", "error") if x in e} for name, e in v.items()}
+        elif v is not None or k == "vs_baseline":
+            out[k] = v
+
+    def rounded(v):
+        if isinstance(v, float):
+            return float(f"{v:.6g}")
+        if isinstance(v, dict):
+            return {k: rounded(x) for k, x in v.items()}
+        return v
+    keep = {k: out[k] for k in ("value", "ms_per_step", "e2e", "steps", "warmup") if k in out}
+    return {**{k: rounded(v) for k, v in out.items()}, **keep}
+
+
 def main():
     args = parse_args()
     if args.impl == "reference":
@@ -1107,7 +1139,10 @@ def main():
             and args.shape == "512,512,512" and args.precision == "native" and args.dtype == "c64"):
         line["secondary"] = run_secondary(args)
     if line is not None:
-        print(json.dumps(line), flush=True)
+        short = headline(line)
+        if len(json.dumps(short)) < len(json.dumps(line)):
+            print("full record: " + json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(short), flush=True)
     if err:
         print(err, file=sys.stderr)
         sys.exit(1)
