@@ -7,7 +7,7 @@ the whole hot path in each direction.  Inputs (1 GiB) are larger than L2
 B_alg = 4 * N * 8 bytes per transform (one round trip for phase A, one for
 phase B), divided by the measured time.
 
-Prints one JSON line (rank 0).  With --impl reference it times the FP64 CPU
+Prints one JSON line (rank 0), the figures; the full record goes to stderr.  With --impl reference it times the FP64 CPU
 oracle instead (the reference arm of this single-GPU tier).
 Under torchrun with N > 1, every rank runs its own replica (no collective on
 the data path; the method's single all-to-all is not exercised on one node of

@@ -436,7 +436,7 @@ __device__ __forceinline__ bool fx_stage(longlong2 *sm, const int4 *__restrict__
     return true;
 }
 
-// The FP64 form of the stages and the store, for a tile that cannot be scaled.
+// The FP64 form of the stages and the store, for a tile with an infinity or NaN, and lines of one point.
 template <int DIR, int R0>
 __device__ __noinline__ void axis_finish_fp64(const AxisPass &a, const AxisOrigin &o, double2 *sm, double2 *dst,
                                               const double2 *tw) {

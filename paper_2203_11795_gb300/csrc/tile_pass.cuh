@@ -23,7 +23,7 @@
 // the stages' accesses without bank conflicts.
 //
 // Arithmetic: FP32 (complex64); for complex128 fixed point (fixed64.cuh) with one exponent per sub-DFT, and a tile with
-// values that cannot be scaled is run again in FP64 from its input.
+// an infinity or NaN is run again in FP64 from its input.
 #pragma once
 
 #include <cuda_runtime.h>
